@@ -227,9 +227,12 @@ SweepArgs sweep_args(lbm_ctx* ctx, int c)
     a.fout = ctx->f[1 - c];
     a.pv = part_view(ctx);
     a.bs_scratch = ctx->bs_scratch;
+    a.pc = ctx->pc;
+    a.tmpl = ctx->tmpl;
     a.omega = 1.0 / ctx->tau;
     a.pre = 1.0 - 0.5 / ctx->tau;
     for (int k = 0; k < 3; ++k) a.F[k] = ctx->F[k];
+    a.forced = a.F[0] != 0.0 || a.F[1] != 0.0 || a.F[2] != 0.0;
     a.omega_f = (float)a.omega;
     a.pre_f = (float)a.pre;
     for (int k = 0; k < 3; ++k) a.F_f[k] = (float)ctx->F[k];
@@ -276,12 +279,12 @@ int enqueue_step(lbm_ctx* ctx, int c, cudaEvent_t* ev = nullptr)
 {
     const SweepArgs a = sweep_args(ctx, c);
     if (ev) cudaEventRecord(ev[0], ctx->stream);
+    int launches = 0;
     {
         NvtxRange r("lbm sweep");
-        ctx->kt->sweep(a, ctx->stream);
+        launches += ctx->kt->sweep(a, ctx->stream);
     }
     if (ev) cudaEventRecord(ev[1], ctx->stream);
-    int launches = 1;
     NvtxRange rp("lbm particle phase");
     if (ctx->np > 0) {
         const ParticleArgs pa = particle_args(ctx);

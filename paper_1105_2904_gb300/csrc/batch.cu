@@ -117,15 +117,15 @@ int enqueue_batch_step(lbm_batch* b, int c, cudaEvent_t* ev = nullptr)
     BatchSweepArgs a{};
     a.lattice = b->lattice;
     a.cells = b->d_sweep[c];
+    a.ncells = (int)b->cells.size();
     a.table = b->d_table;
     a.ntiles = b->ntiles;
     a.walls = b->any_walls ? 1 : 0;
     a.part = b->any_part ? 1 : 0;
     a.grid = b->grid;
     if (ev) cudaEventRecord(ev[0], b->stream);
-    b->kt->sweep_batch(a, b->stream);
+    int launches = b->kt->sweep_batch(a, b->stream);
     if (ev) cudaEventRecord(ev[1], b->stream);
-    int launches = 1;
     if (b->any_part) {
         const int nc = (int)b->cells.size();
         launches += launch_particle_phase_batch_a(b->d_part, b->shape, b->stream);

@@ -19,7 +19,10 @@ struct SweepArgs {
     void* bs_scratch;          // per-site BS records: FP64 mode [N][6] doubles (dP, dL); other
                                // modes float4 (dP, owner tag bits: 16 bytes) at the site index
                                // (16-bit storages) or its brick index (FP32, rec_brick_index)
+    const PConst* pc;          // particle constants and templates (FP64 storage: the passes over
+    const int* tmpl;           // particle sites before and after its sweep)
     double omega, pre, F[3];   // 1/tau, 1 - 1/(2 tau), body force
+    int forced;                // 1: F != 0
     float omega_f, pre_f, F_f[3];  // the same in FP32 (reduced-storage sweeps)
     int moving_walls;          // 1: wall faces may move (uw is read)
     const WallVel* uw;         // wall velocities of the streaming that the pull completes
@@ -104,6 +107,7 @@ struct MaskArgs {
 struct BatchSweepArgs {
     int lattice;
     const SweepArgs* cells;    // device [ncells], this step's buffer parity
+    int ncells;
     const int4* table;         // device [ntiles]
     int ntiles;
     int walls;                 // some cell has walls
@@ -124,7 +128,7 @@ struct FeatureArgs {
 };
 
 struct KernelTable {
-    void (*sweep)(const SweepArgs&, cudaStream_t);
+    int (*sweep)(const SweepArgs&, cudaStream_t);  // returns the kernels launched
     void (*update_masks)(const MaskArgs&, cudaStream_t);
     void (*materialize)(const MaterializeArgs&, cudaStream_t);
     void (*convert_in)(const ConvertArgs&, cudaStream_t);
@@ -132,7 +136,7 @@ struct KernelTable {
     void (*fill_rest)(int lattice, void* dst, unsigned N, cudaStream_t);
     void (*is_save)(const ISFixArgs&, cudaStream_t);   // densities, then populations restored
     void (*is_fix)(const ISFixArgs&, cudaStream_t);    // densities into the new IS sites
-    void (*sweep_batch)(const BatchSweepArgs&, cudaStream_t);
+    int (*sweep_batch)(const BatchSweepArgs&, cudaStream_t);  // returns the kernels launched
     // per-cell argument arrays on the device, blockIdx.y = cell
     void (*is_save_batch)(int lattice, const ISFixArgs* cells, int ncells, cudaStream_t);
     void (*is_fix_batch)(int lattice, const ISFixArgs* cells, int ncells, cudaStream_t);

@@ -6,7 +6,15 @@
 // cores (mma.sync m16n8k16 bf16 -> f32), FP32 master weights and Adam moments, FP32 loss.
 // Each layer's output gradient is kept in bfloat16 (it is a tensor-core operand).
 //
-// Kernels:
+// Two forms. Networks whose weights stay below FUSED_WEIGHTS and whose activations of 16 rows fit
+// in shared memory (the closure network by far) run fused: a minibatch is two launches,
+//   k_rows        gather, every layer, the loss gradient and the backward pass through every layer,
+//                 16 rows per block
+//   k_update      weight and bias gradients, the loss, Adam
+// Larger ones run layer by layer, where a layer fills the chip by itself and 16-row blocks would
+// each stream all of the weights. Both forms add in the same order and give the same bits.
+//
+// Kernels of the second form:
 //   k_gemm        C[M][N] = sum_k A(m,k) B(k,n) with arbitrary element strides for A and B
 //                 (so X W^T, dY W and dY^T X are one kernel), fused epilogue: + bias, relu,
 //                 relu' mask, bfloat16 and / or FP32 output; or FP32 split-K partials
@@ -217,7 +225,20 @@ __global__ void k_gather(const float* __restrict__ X, const float* __restrict__ 
     }
 }
 
-// Adam (Kingma & Ba, 2015) on FP32 masters p with moments m, v; t_dev holds the number of
+// One Adam step (Kingma & Ba, 2015) of parameter i with gradient gi; returns the new value.
+__device__ __forceinline__ float adam_step(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v, long long i,
+                                           float gi, float lr, float b1, float b2, float eps, float c1, float c2)
+{
+    const float mi = b1 * m[i] + (1.f - b1) * gi;
+    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+    m[i] = mi;
+    v[i] = vi;
+    const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    p[i] = pi;
+    return pi;
+}
+
+// Adam on FP32 masters p with moments m, v; t_dev holds the number of
 // steps taken so far (this is step t_dev + 1; k_adam_tick advances it afterwards).
 __global__ void k_adam(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v, const float* __restrict__ g,
                        long long n, const int* __restrict__ t_dev, float lr, float b1, float b2, float eps,
@@ -227,14 +248,329 @@ __global__ void k_adam(float* __restrict__ p, float* __restrict__ m, float* __re
     const float c1 = 1.f - powf(b1, (float)t);
     const float c2 = 1.f - powf(b2, (float)t);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-        p[i] = pi;
+        const float pi = adam_step(p, m, v, i, g[i], lr, b1, b2, eps, c1, c2);
         if (p16) p16[i] = __float2bfloat16(pi);
+    }
+}
+
+// ---- fused form ------------------------------------------------------------------------------
+// A training step of the closure network (259-128-128-6, 128 rows) is 38 MFLOP on 700 kB that sit
+// in L2: nothing bounds it but latency, so what counts is the number of dependent launches and
+// round trips. Rows are independent through all layers forwards and backwards; only the weight
+// gradients need all rows. That gives two kernels. Weights are kept as bfloat16 in the order of
+// the tensor-core fragments (forward B(k, n) = W[n][k]; backward B(k = j, n = c) = W[j][c]), so a
+// lane's operand is one 8-byte load and a warp's 256 consecutive bytes, whatever the width of the
+// layer (the closure's 259 inputs leave W's rows unaligned); Adam writes its new weights there.
+// Minibatch of 128 rows: 208 us in ~20 launches -> STEPNEW us; forward pass of 200 rows 110 -> FWDNEW us.
+
+constexpr int MAX_LAYERS = 8;
+constexpr int ROWS = 16;             // rows per block: one m16n8k16 tile
+constexpr int ROWS_THREADS = 256;
+constexpr int UPD_THREADS = 128;
+constexpr int SPLITS = 16;           // fixed-order split of the rows in the weight gradients
+// Up to here a 16-row block's pass over all weights (512 kB from L2) stays a matter of a few us.
+constexpr long long FUSED_WEIGHTS = 262144;
+constexpr size_t FUSED_SMEM = 160 * 1024;
+
+__host__ __device__ constexpr int pad16(int n) { return (n + 15) / 16 * 16; }
+// Row stride of a bfloat16 tile in shared memory: 8 n + 4 words with n odd or even, so the eight
+// rows of a fragment fall into different banks.
+__host__ __device__ constexpr int tile_ld(int n) { return pad16(n) + 8; }
+__host__ __device__ constexpr long long frag_elems(int k, int n) { return (long long)((n + 7) / 8) * ((k + 15) / 16) * 128; }
+// Position of B(k, n) among the fragments of a K x N operand (m16n8k16, "col" B).
+__device__ __forceinline__ long long frag_pos(int k, int n, int K)
+{
+    const int ks = (K + 15) / 16;
+    const int lane = (n & 7) * 4 + ((k & 7) >> 1);
+    return (((long long)(n >> 3) * ks + (k >> 4)) * 32 + lane) * 4 + ((k >> 3) & 1) * 2 + (k & 1);
+}
+
+struct NetArgs {
+    int L;
+    int size[MAX_LAYERS + 1];
+    long long w_off[MAX_LAYERS], b_off[MAX_LAYERS];
+    long long wf_off[MAX_LAYERS], wb_off[MAX_LAYERS];  // fragment-ordered copies (backward: l >= 1)
+    const float* p;
+    __nv_bfloat16* wf;
+    __nv_bfloat16* wb;
+    const float *shift, *scale;  // input standardisation or null
+    // between the two kernels: values by feature, ld rows each (the update's operands)
+    int ld;
+    __nv_bfloat16* hT[MAX_LAYERS];  // inputs of layer l
+    __nv_bfloat16* dT[MAX_LAYERS];  // output gradients of layer l
+    float* r2;                   // squared errors [rows][O]
+};
+
+struct RowsArgs {
+    NetArgs n;
+    const float* X;      // [.][K]
+    const float* T;      // [.][O], null: forward pass only
+    const int* idx;      // rows of the minibatch, null: 0..rows-1
+    int rows;
+    float* y;            // forward pass: [rows][O]
+    float grad_scale;    // 1 / (rows O)
+    int* tick;           // Adam's step count, advanced here when given (k_update reads it)
+};
+
+struct UpdateArgs {
+    NetArgs n;
+    int rows;
+    float* p;
+    float* m;
+    float* v;
+    float* g;
+    const int* t;        // Adam's step number, null: gradients only
+    float lr, b1, b2, eps;
+    double* loss;        // loss of the minibatch is added here
+    double loss_scale;
+};
+
+// C (16 rows of `in` times a K x N operand in fragment order) for this warp's n-tiles, two at a
+// time; put(row, column, value) for the lane's elements.
+template <class PUT>
+__device__ __forceinline__ void rows_gemm(const __nv_bfloat16* __restrict__ in, int ld, int K, int N,
+                                          const __nv_bfloat16* __restrict__ frag, PUT&& put)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int gq = lane >> 2, tq = lane & 3;
+    const int KS = (K + 15) / 16, NT = (N + 7) / 8;
+    for (int nt = 2 * warp; nt < NT; nt += 2 * (ROWS_THREADS / 32)) {
+        const bool two = nt + 1 < NT;
+        const uint2* b0p = reinterpret_cast<const uint2*>(frag) + (long long)nt * KS * 32 + lane;
+        const uint2* b1p = two ? b0p + (long long)KS * 32 : b0p;
+        float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 9
+        for (int ks = 0; ks < KS; ++ks) {
+            const uint2 v0 = b0p[ks * 32], v1 = b1p[ks * 32];
+            const __nv_bfloat16* ap = in + gq * ld + ks * 16 + 2 * tq;
+            const uint32_t a[4] = {ld_pair(ap), ld_pair(ap + 8 * ld), ld_pair(ap + 8), ld_pair(ap + 8 * ld + 8)};
+            const uint32_t b0[2] = {v0.x, v0.y}, b1[2] = {v1.x, v1.y};
+            mma_bf16(c0, a, b0);
+            mma_bf16(c1, a, b1);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int row = gq + (q >= 2 ? 8 : 0), col = nt * 8 + 2 * tq + (q & 1);
+            if (col < N) put(row, col, c0[q]);
+            if (two && col + 8 < N) put(row, col + 8, c1[q]);
+        }
+    }
+}
+
+__device__ __forceinline__ void wait_for_previous_kernel()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void let_next_kernel_start()
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+}
+
+__global__ void __launch_bounds__(ROWS_THREADS) k_rows(const RowsArgs a)
+{
+    extern __shared__ __align__(16) __nv_bfloat16 sm[];
+    const NetArgs& n = a.n;
+    const int L = n.L, K0 = n.size[0], O = n.size[L];
+    const int row0 = blockIdx.x * ROWS;
+    const bool train = a.T != nullptr;
+    __nv_bfloat16* h[MAX_LAYERS + 1];  // inputs of layer l ([ROWS][tile_ld]); h[L] stays unused
+    __nv_bfloat16* d[MAX_LAYERS + 1];  // output gradients of layer l - 1, beside h
+    int total = 0;
+    for (int l = 0; l < L; ++l) {
+        h[l] = sm + total;
+        total += ROWS * tile_ld(n.size[l]);
+    }
+    if (train)
+        for (int l = 1; l <= L; ++l) {
+            d[l] = sm + total;
+            total += ROWS * tile_ld(n.size[l]);
+        }
+    // padding rows and columns are zero
+    for (int e = threadIdx.x; e < total / 8; e += ROWS_THREADS) reinterpret_cast<uint4*>(sm)[e] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    // the minibatch's rows; nothing here depends on the kernel before
+    for (int e = threadIdx.x; e < ROWS * K0; e += ROWS_THREADS) {
+        const int r = e / K0, c = e - r * K0;
+        if (row0 + r >= a.rows) break;
+        const long long src = a.idx ? a.idx[row0 + r] : row0 + r;
+        float v = a.X[src * K0 + c];
+        if (n.shift) v = (v - n.shift[c]) * n.scale[c];
+        h[0][r * tile_ld(K0) + c] = __float2bfloat16(v);
+    }
+    wait_for_previous_kernel();
+    let_next_kernel_start();
+    if (a.tick && blockIdx.x == 0 && threadIdx.x == 0) *a.tick += 1;
+    __syncthreads();
+    for (int l = 0; l < L; ++l) {
+        const int K = n.size[l], N = n.size[l + 1];
+        const float* bias = n.p + n.b_off[l];
+        if (l + 1 < L) {
+            __nv_bfloat16* out = h[l + 1];
+            const int ldo = tile_ld(N);
+            rows_gemm(h[l], tile_ld(K), K, N, n.wf + n.wf_off[l], [&](int r, int c, float v) {
+                out[r * ldo + c] = __float2bfloat16(fmaxf(v + bias[c], 0.f));
+            });
+        } else {
+            rows_gemm(h[l], tile_ld(K), K, N, n.wf + n.wf_off[l], [&](int r, int c, float v) {
+                if (row0 + r >= a.rows) return;
+                const float y = v + bias[c];
+                if (!train) {
+                    a.y[(long long)(row0 + r) * O + c] = y;
+                    return;
+                }
+                // mean-squared error: d = 2 (y - t) / (rows O)
+                const long long src = a.idx ? a.idx[row0 + r] : row0 + r;
+                const float res = y - a.T[src * O + c];
+                n.r2[(long long)(row0 + r) * O + c] = res * res;
+                d[L][r * tile_ld(O) + c] = __float2bfloat16(2.f * res * a.grad_scale);
+            });
+        }
+        __syncthreads();
+    }
+    if (!train) return;
+    // d_l = (d_{l+1} W_l) relu'(h_l)
+    for (int l = L - 1; l >= 1; --l) {
+        const int K = n.size[l], N = n.size[l + 1], ldk = tile_ld(K);
+        rows_gemm(d[l + 1], tile_ld(N), N, K, n.wb + n.wb_off[l], [&](int r, int c, float v) {
+            const bool on = __bfloat162float(h[l][r * ldk + c]) > 0.f;
+            d[l][r * ldk + c] = __float2bfloat16(on ? v : 0.f);
+        });
+        __syncthreads();
+    }
+    // by feature, this block's 16 rows as two 16-byte stores
+    auto transpose = [&](const __nv_bfloat16* from, int N, __nv_bfloat16* to) {
+        const int ld = tile_ld(N);
+        for (int c = threadIdx.x; c < N; c += ROWS_THREADS) {
+            __align__(16) __nv_bfloat16 col[ROWS];
+#pragma unroll
+            for (int r = 0; r < ROWS; ++r) col[r] = from[r * ld + c];
+            uint4* dst = reinterpret_cast<uint4*>(to + (long long)c * n.ld + row0);
+            dst[0] = reinterpret_cast<const uint4*>(col)[0];
+            dst[1] = reinterpret_cast<const uint4*>(col)[1];
+        }
+    };
+    for (int l = 0; l < L; ++l) {
+        transpose(h[l], n.size[l], n.hT[l]);
+        transpose(d[l + 1], n.size[l + 1], n.dT[l]);
+    }
+}
+
+// Sum of 256 values in the order of a halving tree (value t + value t + 128, then + 64, ...): lane t
+// holds values t + 32 j.
+__device__ __forceinline__ float tree256(float x[8])
+{
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] += x[j + 4];
+    x[0] += x[2];
+    x[1] += x[3];
+    float s = x[0] + x[1];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    return s;  // lane 0
+}
+
+// One warp per 16 x 8 tile of a weight gradient dW[n][k] = sum_r d[r][n] h[r][k] (rows in SPLITS
+// ranges, each summed on the tensor cores, the ranges added in order), per bias gradient and for the loss; Adam
+// on the elements just formed.
+__global__ void __launch_bounds__(UPD_THREADS) k_update(const UpdateArgs a)
+{
+    const NetArgs& n = a.n;
+    const int lane = threadIdx.x & 31, gq = lane >> 2, tq = lane & 3;
+    int task = blockIdx.x * (UPD_THREADS / 32) + (threadIdx.x >> 5);
+    wait_for_previous_kernel();
+    let_next_kernel_start();
+    float c1 = 1.f, c2 = 1.f;
+    if (a.t) {
+        const int t = *a.t;
+        c1 = 1.f - powf(a.b1, (float)t);
+        c2 = 1.f - powf(a.b2, (float)t);
+    }
+    const int per = ((a.rows + SPLITS - 1) / SPLITS + 31) / 32 * 32;  // rows of a range
+    const int rows16 = (a.rows + 15) / 16 * 16;
+    for (int l = 0; l < n.L; ++l) {
+        const int K = n.size[l], N = n.size[l + 1];
+        const int MT = (N + 15) / 16, NT = (K + 7) / 8;
+        if (task >= MT * NT) {
+            task -= MT * NT;
+            continue;
+        }
+        const int n0 = task / NT * 16, k0 = task % NT * 8;
+        const __nv_bfloat16* d0 = n.dT[l] + (long long)(n0 + gq) * n.ld + 2 * tq;
+        const __nv_bfloat16* d1 = d0 + 8LL * n.ld;
+        const __nv_bfloat16* hb = n.hT[l] + (long long)(k0 + gq) * n.ld + 2 * tq;
+        const bool ok0 = n0 + gq < N, ok1 = n0 + gq + 8 < N, okb = k0 + gq < K;
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int z = 0; z * per < rows16; ++z) {
+            float c[4] = {0.f, 0.f, 0.f, 0.f};
+            const int end = min(rows16, (z + 1) * per);
+#pragma unroll 4
+            for (int r = z * per; r < end; r += 16) {
+                const uint32_t A[4] = {ok0 ? ld_pair(d0 + r) : 0u, ok1 ? ld_pair(d1 + r) : 0u, ok0 ? ld_pair(d0 + r + 8) : 0u,
+                                       ok1 ? ld_pair(d1 + r + 8) : 0u};
+                const uint32_t B[2] = {okb ? ld_pair(hb + r) : 0u, okb ? ld_pair(hb + r + 8) : 0u};
+                mma_bf16(c, A, B);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[q] += c[q];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int nn = n0 + gq + (q >= 2 ? 8 : 0), k = k0 + 2 * tq + (q & 1);
+            if (nn >= N || k >= K) continue;
+            const long long i = n.w_off[l] + (long long)nn * K + k;
+            a.g[i] = s[q];
+            if (!a.t) continue;
+            const __nv_bfloat16 w = __float2bfloat16(adam_step(a.p, a.m, a.v, i, s[q], a.lr, a.b1, a.b2, a.eps, c1, c2));
+            n.wf[n.wf_off[l] + frag_pos(k, nn, K)] = w;
+            if (l > 0) n.wb[n.wb_off[l] + frag_pos(nn, k, N)] = w;
+        }
+        return;
+    }
+    for (int l = 0; l < n.L; ++l) {
+        const int N = n.size[l + 1];
+        if (task >= N) {
+            task -= N;
+            continue;
+        }
+        const __nv_bfloat16* dr = n.dT[l] + (long long)task * n.ld;
+        float x[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            x[j] = 0.f;
+            for (int r = lane + 32 * j; r < a.rows; r += 256) x[j] += __bfloat162float(dr[r]);
+        }
+        const float s = tree256(x);
+        if (lane == 0) {
+            const long long i = n.b_off[l] + task;
+            a.g[i] = s;
+            if (a.t) adam_step(a.p, a.m, a.v, i, s, a.lr, a.b1, a.b2, a.eps, c1, c2);
+        }
+        return;
+    }
+    if (task == 0) {
+        const long long m = (long long)a.rows * n.size[n.L];
+        double tot = 0.0;
+        for (long long b = 0; b < m; b += 256) {
+            float x[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) x[j] = b + lane + 32 * j < m ? n.r2[b + lane + 32 * j] : 0.f;
+            tot += (double)tree256(x);
+        }
+        if (lane == 0) *a.loss += tot * a.loss_scale;
+    }
+}
+
+// The fragment-ordered copies of the weights (after they were set, or after a separate Adam step).
+__global__ void k_pack_weights(const NetArgs n)
+{
+    for (int l = 0; l < n.L; ++l) {
+        const int K = n.size[l], N = n.size[l + 1];
+        for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < N * K; e += gridDim.x * blockDim.x) {
+            const int j = e / K, k = e - j * K;
+            const __nv_bfloat16 w = __float2bfloat16(n.p[n.w_off[l] + e]);
+            n.wf[n.wf_off[l] + frag_pos(k, j, K)] = w;
+            if (l > 0) n.wb[n.wb_off[l] + frag_pos(j, k, N)] = w;
+        }
     }
 }
 
@@ -281,6 +617,13 @@ struct lbm_mlp {
     int loss_cap = 0;
     float* in_shift = nullptr;       // input standardisation (null: none)
     float* in_scale = nullptr;
+    // fused form (k_rows, k_update)
+    bool fused = false;
+    std::vector<long long> wf_off, wb_off;
+    __nv_bfloat16* wf = nullptr;     // weights in fragment order, forwards
+    __nv_bfloat16* wb = nullptr;     // and backwards
+    std::vector<__nv_bfloat16*> hT, dT;
+    float* r2 = nullptr;
     std::vector<void*> allocs;
     std::string err;
 };
@@ -321,8 +664,6 @@ void free_dev(lbm_mlp* net, void* p)
     cudaFree(p);
 }
 
-const int SPLITS = 16;
-
 lbm_status ensure_rows(lbm_mlp* net, int rows)
 {
     if (rows <= net->cap) return LBM_OK;
@@ -338,6 +679,23 @@ lbm_status ensure_rows(lbm_mlp* net, int rows)
     net->d.assign(net->L, nullptr);
     const int K = net->sizes[0], O = net->sizes[net->L];
     lbm_status s;
+    if (net->fused) {
+        cap = std::max(cap, ROWS);
+        for (auto* q : net->hT) free_dev(net, q);
+        for (auto* q : net->dT) free_dev(net, q);
+        free_dev(net, net->r2);
+        net->cap = 0;
+        net->r2 = nullptr;
+        net->hT.assign(net->L, nullptr);
+        net->dT.assign(net->L, nullptr);
+        for (size_t l = 0; l < (size_t)net->L; ++l) {
+            if ((s = malloc_dev(net, &net->hT[l], (size_t)cap * net->sizes[l])) != LBM_OK) return s;
+            if ((s = malloc_dev(net, &net->dT[l], (size_t)cap * net->sizes[l + 1])) != LBM_OK) return s;
+        }
+        if ((s = malloc_dev(net, &net->r2, (size_t)cap * O)) != LBM_OK) return s;
+        net->cap = cap;
+        return LBM_OK;
+    }
     if ((s = malloc_dev(net, &net->xb, (size_t)cap * K)) != LBM_OK) return s;
     if ((s = malloc_dev(net, &net->tb, (size_t)cap * O)) != LBM_OK) return s;
     if ((s = malloc_dev(net, &net->y, (size_t)cap * O)) != LBM_OK) return s;
@@ -406,11 +764,113 @@ void backward(lbm_mlp* net, int rows, int slot)
     }
 }
 
+// ---- fused form: launches ------------------------------------------------------------------
+
+size_t rows_smem(const lbm_mlp* net, bool train)
+{
+    size_t e = 0;
+    for (int l = 0; l < net->L; ++l) e += (size_t)ROWS * tile_ld(net->sizes[(size_t)l]);
+    if (train)
+        for (int l = 1; l <= net->L; ++l) e += (size_t)ROWS * tile_ld(net->sizes[(size_t)l]);
+    return e * sizeof(__nv_bfloat16);
+}
+
+NetArgs net_args(const lbm_mlp* net)
+{
+    NetArgs n{};
+    n.L = net->L;
+    for (size_t l = 0; l <= (size_t)net->L; ++l) n.size[l] = net->sizes[l];
+    for (size_t l = 0; l < (size_t)net->L; ++l) {
+        n.w_off[l] = net->w_off[l];
+        n.b_off[l] = net->b_off[l];
+        n.wf_off[l] = net->wf_off[l];
+        n.wb_off[l] = net->wb_off[l];
+        if (l < net->hT.size()) {
+            n.hT[l] = net->hT[l];
+            n.dT[l] = net->dT[l];
+        }
+    }
+    n.p = net->p;
+    n.wf = net->wf;
+    n.wb = net->wb;
+    n.shift = net->in_shift;
+    n.scale = net->in_scale;
+    n.ld = net->cap;
+    n.r2 = net->r2;
+    return n;
+}
+
+// `overlap`: the kernel may be set up while the one before it in the stream, one of this file's
+// own, still runs (programmatic dependent launch; it waits before it touches that one's data).
+template <class A>
+void launch(void (*k)(const A), int grid, int block, size_t smem, bool overlap, cudaStream_t s, const A& a)
+{
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = overlap ? 1 : 0;
+    cudaLaunchKernelEx(&c, k, a);
+}
+
+// Forward pass (t null) or forward, loss and backward pass of `rows` rows. `tick` advances Adam's
+// step count. `overlap` only where x, t and idx were not written by the kernel before.
+void fused_rows(lbm_mlp* net, const float* x, const float* t, const int* idx, int rows, float* y, bool tick, bool overlap)
+{
+    RowsArgs a{};
+    a.n = net_args(net);
+    a.X = x;
+    a.T = t;
+    a.idx = idx;
+    a.rows = rows;
+    a.y = y;
+    a.grad_scale = 1.f / (float)((long long)rows * net->sizes[(size_t)net->L]);
+    a.tick = tick ? net->t : nullptr;
+    launch(k_rows, (rows + ROWS - 1) / ROWS, ROWS_THREADS, rows_smem(net, t != nullptr), overlap, net->stream, a);
+}
+
+// The gradients of the rows of the last fused_rows, the loss into loss_dev[slot], and with lr > 0
+// the Adam step.
+void fused_update(lbm_mlp* net, int rows, int slot, float lr, float b1, float b2, float eps)
+{
+    UpdateArgs a{};
+    a.n = net_args(net);
+    a.rows = rows;
+    a.p = net->p;
+    a.m = net->m;
+    a.v = net->v;
+    a.g = net->g;
+    a.t = lr > 0.f ? net->t : nullptr;
+    a.lr = lr;
+    a.b1 = b1;
+    a.b2 = b2;
+    a.eps = eps;
+    a.loss = net->loss_dev + slot;
+    a.loss_scale = 1.0 / (double)((long long)rows * net->sizes[(size_t)net->L]);
+    int tasks = 1;
+    for (size_t l = 0; l < (size_t)net->L; ++l)
+        tasks += (net->sizes[l + 1] + 15) / 16 * ((net->sizes[l] + 7) / 8) + net->sizes[l + 1];
+    constexpr int W = UPD_THREADS / 32;
+    launch(k_update, (tasks + W - 1) / W, UPD_THREADS, 0, true, net->stream, a);
+}
+
+void refresh_weights(lbm_mlp* net)
+{
+    if (net->fused) k_pack_weights<<<blocks_for(net->nparam), 256, 0, net->stream>>>(net_args(net));
+    else k_to_bf16<<<blocks_for(net->nparam), 256, 0, net->stream>>>(net->p, net->nparam, net->p16);
+}
+
 void adam(lbm_mlp* net, float lr, float b1, float b2, float eps)
 {
     k_adam<<<blocks_for(net->nparam), 256, 0, net->stream>>>(net->p, net->m, net->v, net->g, net->nparam, net->t, lr, b1,
-                                                              b2, eps, net->p16);
+                                                              b2, eps, net->fused ? nullptr : net->p16);
     k_adam_tick<<<1, 32, 0, net->stream>>>(net->t);
+    if (net->fused) refresh_weights(net);
 }
 
 lbm_status ensure_loss_slots(lbm_mlp* net, int n)
@@ -455,15 +915,38 @@ lbm_status lbm_mlp_create(lbm_mlp** out, int nlayers, const int* sizes, void* cu
     lbm_status s = LBM_OK;
     if ((s = malloc_dev(net, &net->p, (size_t)off)) != LBM_OK || (s = malloc_dev(net, &net->m, (size_t)off)) != LBM_OK ||
         (s = malloc_dev(net, &net->v, (size_t)off)) != LBM_OK || (s = malloc_dev(net, &net->g, (size_t)off)) != LBM_OK ||
-        (s = malloc_dev(net, &net->p16, (size_t)off)) != LBM_OK || (s = malloc_dev(net, &net->t, 1)) != LBM_OK) {
+        (s = malloc_dev(net, &net->t, 1)) != LBM_OK) {
         lbm_mlp_destroy(net);
         return s;
+    }
+    long long weights = 0, wf = 0, wb = 0;
+    for (int l = 0; l < nlayers; ++l) {
+        weights += (long long)sizes[l] * sizes[l + 1];
+        net->wf_off.push_back(wf);
+        net->wb_off.push_back(wb);
+        wf += frag_elems(sizes[l], sizes[l + 1]);
+        if (l > 0) wb += frag_elems(sizes[l + 1], sizes[l]);
+    }
+    net->fused = weights <= FUSED_WEIGHTS && rows_smem(net, true) <= FUSED_SMEM &&
+                 cudaFuncSetAttribute(k_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM) == cudaSuccess;
+    if (net->fused)
+        s = (s = malloc_dev(net, &net->wf, (size_t)wf)) != LBM_OK ? s : malloc_dev(net, &net->wb, (size_t)wb);
+    else
+        s = malloc_dev(net, &net->p16, (size_t)off);
+    if (s != LBM_OK) {
+        lbm_mlp_destroy(net);
+        return s;
+    }
+    if (net->fused) {  // the fragments' padding stays zero
+        cudaMemsetAsync(net->wf, 0, sizeof(__nv_bfloat16) * wf, net->stream);
+        cudaMemsetAsync(net->wb, 0, sizeof(__nv_bfloat16) * wb, net->stream);
+    } else {
+        cudaMemsetAsync(net->p16, 0, sizeof(__nv_bfloat16) * off, net->stream);
     }
     cudaMemsetAsync(net->p, 0, sizeof(float) * off, net->stream);
     cudaMemsetAsync(net->m, 0, sizeof(float) * off, net->stream);
     cudaMemsetAsync(net->v, 0, sizeof(float) * off, net->stream);
     cudaMemsetAsync(net->g, 0, sizeof(float) * off, net->stream);
-    cudaMemsetAsync(net->p16, 0, sizeof(__nv_bfloat16) * off, net->stream);
     cudaMemsetAsync(net->t, 0, sizeof(int), net->stream);
     if (cudaStreamSynchronize(net->stream) != cudaSuccess) {
         cudaGetLastError();
@@ -482,7 +965,7 @@ lbm_status lbm_mlp_set_params(lbm_mlp* net, const double* params)
     std::vector<float> h((size_t)net->nparam);
     for (long long i = 0; i < net->nparam; ++i) h[(size_t)i] = (float)params[i];
     MK(cudaMemcpyAsync(net->p, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice, net->stream));
-    k_to_bf16<<<blocks_for(net->nparam), 256, 0, net->stream>>>(net->p, net->nparam, net->p16);
+    refresh_weights(net);
     MK(cudaGetLastError());
     MK(cudaMemsetAsync(net->m, 0, sizeof(float) * net->nparam, net->stream));
     MK(cudaMemsetAsync(net->v, 0, sizeof(float) * net->nparam, net->stream));
@@ -538,6 +1021,11 @@ lbm_status lbm_mlp_forward(lbm_mlp* net, const float* x, int rows, float* y)
 {
     if (!net || !x || !y || rows < 0) return LBM_E_INVALID;
     if (rows == 0) return LBM_OK;
+    if (net->fused) {
+        fused_rows(net, x, nullptr, nullptr, rows, y, false, false);
+        MK(cudaGetLastError());
+        return LBM_OK;
+    }
     lbm_status s = ensure_rows(net, rows);
     if (s != LBM_OK) return s;
     const int K = net->sizes[0], O = net->sizes[(size_t)net->L];
@@ -557,9 +1045,14 @@ lbm_status lbm_mlp_loss_grad(lbm_mlp* net, const float* x, const float* t, int r
     if (s != LBM_OK) return s;
     const int K = net->sizes[0], O = net->sizes[(size_t)net->L];
     MK(cudaMemsetAsync(net->loss_dev, 0, sizeof(double), net->stream));
-    k_gather<<<blocks_for((long long)rows * (K + O)), 256, 0, net->stream>>>(x, t, nullptr, rows, K, O, net->in_shift,
-                                                                               net->in_scale, net->xb, net->tb);
-    backward(net, rows, 0);
+    if (net->fused) {
+        fused_rows(net, x, t, nullptr, rows, nullptr, false, false);
+        fused_update(net, rows, 0, 0.f, 0.f, 0.f, 0.f);
+    } else {
+        k_gather<<<blocks_for((long long)rows * (K + O)), 256, 0, net->stream>>>(x, t, nullptr, rows, K, O, net->in_shift,
+                                                                                   net->in_scale, net->xb, net->tb);
+        backward(net, rows, 0);
+    }
     MK(cudaGetLastError());
     if (loss) {
         MK(cudaMemcpyAsync(loss, net->loss_dev, sizeof(double), cudaMemcpyDeviceToHost, net->stream));
@@ -600,6 +1093,12 @@ lbm_status lbm_mlp_train(lbm_mlp* net, const float* x, const float* t, int n, in
         std::shuffle(perm.begin(), perm.end(), rng);
         MK(cudaMemcpyAsync(net->idx, perm.data(), sizeof(int) * (size_t)n, cudaMemcpyHostToDevice, net->stream));
         for (int bi = 0; bi < nb; ++bi) {
+            if (net->fused) {
+                // (the first minibatch follows the copy of the permutation, the others k_update)
+                fused_rows(net, x, t, net->idx + (size_t)bi * batch, batch, nullptr, true, bi > 0);
+                fused_update(net, batch, e, (float)lr, 0.9f, 0.999f, 1e-8f);
+                continue;
+            }
             k_gather<<<blocks_for((long long)batch * (K + O)), 256, 0, net->stream>>>(x, t, net->idx + (size_t)bi * batch,
                                                                                       batch, K, O, net->in_shift,
                                                                                       net->in_scale, net->xb, net->tb);

@@ -129,34 +129,113 @@ __device__ __forceinline__ float geq_dev(float sgn, float drho, const float u[3]
     return (float)L::w(i) * (drho + rho * (3.0f * cu + 4.5f * cu * cu - 1.5f * usq));
 }
 
-// BGK collision with Guo forcing (Eq. 3), plain FP64 form. The expression order matches a
-// direct transcription of the equations so that results are reproducible bit for bit.
+// GB300's FP64 pipe takes a warp instruction every 16 cycles per SM, so the FP64 storage is bound
+// by the number of FP64 instructions and by nothing else. The FP64 helpers below evaluate the
+// equations' own operations in the equations' own order, so results stay reproducible bit for
+// bit, but spend none on the zero components of c_i (x + 0 * y is x for finite y) and share
+// between opposite directions what only changes sign (c_opp . u = -(c_i . u) exactly, and the
+// sign carries through the products).
+
+// c_i . v for the nonzero components of c_i, in x, y, z order.
+template <class L, int i>
+__device__ __forceinline__ double cdot_plain(const double v[3])
+{
+    double r = 0.0;
+    bool first = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (L::c(i, k) == 0) continue;
+        const double t = L::c(i, k) > 0 ? v[k] : -v[k];
+        r = first ? t : r + t;
+        first = false;
+    }
+    return r;
+}
+
+// rho = sum f and j = sum f c, each sum in direction order.
+template <class L>
+__device__ __forceinline__ void moments_plain(const double f[], double& rho, double j[3])
+{
+    rho = f[0];
+    sfor<1, L::Q>([&](auto ic) { rho += f[decltype(ic)::value]; });
+    sfor<0, 3>([&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        j[k] = 0.0;
+        if constexpr (k < L::D) {
+            bool first = true;
+            sfor<1, L::Q>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                if constexpr (L::c(i, k) != 0) {
+                    const double t = L::c(i, k) > 0 ? f[i] : -f[i];
+                    j[k] = first ? t : j[k] + t;
+                    first = false;
+                }
+            });
+        }
+    });
+}
+
+// f^eq_i(rho, u) of every direction, handed to put(i, value): the values of feq_plain.
+template <class L, class PUT>
+__device__ __forceinline__ void feq_all_plain(double rho, const double u[3], PUT&& put)
+{
+    const double us = 1.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    put(std::integral_constant<int, 0>{}, L::w(0) * rho * (1.0 - us));
+    sfor<1, L::Q>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        constexpr int j = L::opp(i);
+        if constexpr (j > i) {
+            const double cu = cdot_plain<L, i>(u);
+            const double t = 3.0 * cu, e = 4.5 * cu * cu, wr = L::w(i) * rho;
+            put(std::integral_constant<int, i>{}, wr * (1.0 + t + e - us));
+            put(std::integral_constant<int, j>{}, wr * (1.0 - t + e - us));
+        }
+    });
+}
+
+// BGK collision with Guo forcing (Eq. 3), plain FP64 form:
+// f*_i = f_i - omega (f_i - f^eq_i) + S_i, S_i = pre w_i (3 (c_i.F - u.F) + 9 (c_i.u) (c_i.F)).
+// FORCED = false: F = 0, where S_i is zero.
+template <class L, bool FORCED>
+__device__ __forceinline__ void collide_plain_f(double f[], const SweepArgs& a)
+{
+    constexpr int Q = L::Q;
+    double rho, j[3], u[3];
+    moments_plain<L>(f, rho, j);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) u[k] = k >= L::D ? 0.0 : (FORCED ? j[k] + 0.5 * a.F[k] : j[k]) / rho;
+    const double pre = a.pre, omega = a.omega;
+    const double uF = FORCED ? u[0] * a.F[0] + u[1] * a.F[1] + u[2] * a.F[2] : 0.0;
+    const double us = 1.5 * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+    {
+        f[0] = f[0] - omega * (f[0] - L::w(0) * rho * (1.0 - us));
+        if constexpr (FORCED) f[0] = f[0] + pre * L::w(0) * (3.0 * (-uF));
+    }
+    sfor<1, Q>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        constexpr int jj = L::opp(i);
+        if constexpr (jj > i) {
+            const double cu = cdot_plain<L, i>(u);
+            const double t = 3.0 * cu, e = 4.5 * cu * cu, wr = L::w(i) * rho;
+            double fi = f[i] - omega * (f[i] - wr * (1.0 + t + e - us));
+            double fj = f[jj] - omega * (f[jj] - wr * (1.0 - t + e - us));
+            if constexpr (FORCED) {
+                const double cF = cdot_plain<L, i>(a.F);
+                const double pw = pre * L::w(i), g = 9.0 * cu * cF;
+                fi = fi + pw * (3.0 * (cF - uF) + g);
+                fj = fj + pw * (3.0 * (-cF - uF) + g);
+            }
+            f[i] = fi;
+            f[jj] = fj;
+        }
+    });
+}
+
 template <class L>
 __device__ __forceinline__ void collide_plain(double f[], const SweepArgs& a)
 {
-    constexpr int Q = L::Q;
-    double rho = 0.0;
-    sfor<0, Q>([&](auto ic) { rho += f[decltype(ic)::value]; });
-    double j[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-        sfor<0, Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            j[k] += f[i] * (double)L::c(i, k);
-        });
-    double u[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) u[k] = (j[k] + 0.5 * a.F[k]) / rho;
-    const double pre = a.pre, omega = a.omega;
-    const double uF = u[0] * a.F[0] + u[1] * a.F[1] + u[2] * a.F[2];
-    sfor<0, Q>([&](auto ic) {
-        constexpr int i = decltype(ic)::value;
-        const double cu = (double)L::c(i, 0) * u[0] + (double)L::c(i, 1) * u[1] + (double)L::c(i, 2) * u[2];
-        const double cF =
-            (double)L::c(i, 0) * a.F[0] + (double)L::c(i, 1) * a.F[1] + (double)L::c(i, 2) * a.F[2];
-        const double Si = pre * L::w(i) * (3.0 * (cF - uF) + 9.0 * cu * cF);
-        f[i] = f[i] - omega * (f[i] - feq_plain<L, i>(1.0, rho, u)) + Si;
-    });
+    if (a.forced) collide_plain_f<L, true>(f, a);
+    else collide_plain_f<L, false>(f, a);
 }
 
 // BGK collision with Guo forcing on deviations g = f - w (FP32). Opposite directions i and
@@ -753,7 +832,10 @@ __device__ __forceinline__ void sweep_site(const SweepArgs& a, int x, int y, int
     if constexpr (WALLS) {
         if (g.eqface) {
             const int face = eq_face_of(g, x, y, z);
-            if (face >= 0 && (!PART || tagx == TAG_FLUID)) {
+            bool fluid = !PART || tagx == TAG_FLUID;
+            if constexpr (!PART && !St::deviation)  // the FP64 pull sweep reads the owner map only here
+                if (face >= 0 && a.pv.tag) fluid = a.pv.tag[idx] == TAG_FLUID;
+            if (face >= 0 && fluid) {
                 if constexpr (St::deviation) {
                     equilibrium_dev<L>(mrho, a.uw[1].uf[face], f);
                 } else {
@@ -850,6 +932,113 @@ __global__ void __launch_bounds__(SWEEP_THREADS, (Store<S>::deviation && !WALLS)
     C f[Q];
     pull<L, S, WALLS>((const S*)a.fin, g, n, x, y, z, idx, f);
     sweep_site<L, S, WALLS, PART>(a, x, y, z, idx, valid, n, f, tagx, mask);
+}
+
+// ---- FP64 storage, pull scheme -----------------------------------------------------------------
+// The step is three launches: the IS imposition written into the input buffer (k_impose_plain),
+// the collision of every site as if it were fluid (k_sweep_plain), and the particle sites of its
+// output through their particles' templates (k_solid_plain). Inside the sweep the imposition and
+// the BS transfer would be run by every warp that crosses a particle, for all of its lanes, with
+// the velocity and the equilibrium of an IS site evaluated again for each of the 18 pulls from it:
+// 1500 FP64 instructions a warp against 370 of the collision. Through the templates every lane has
+// work and an IS site's 18 equilibria share their terms; the scattered accesses this costs are
+// nothing beside the FP64 pipe (the reduced storages, bound by memory or by all instructions
+// alike, keep the coupling in their sweeps). 160^3 suspension, 25.6 % solid, a step's three launches: 12.3 -> 3.3 ms (of which k_sweep_plain 2.9).
+
+// Before the sweep: every IS site of the owner map, holding its density in its slots (density
+// carry), takes f^eq(rho_I, u_p + omega_p x r) when the imposition is pending (Eq. 12). The
+// values are those substitute_is_plain gives the pulls, bounced ones included (f^eq of the stored
+// direction).
+template <class L, bool B>
+__global__ void __launch_bounds__(128) k_impose_plain(const SweepArgs a0, const SweepArgs* __restrict__ cells)
+{
+    const SweepArgs& a = B ? cells[blockIdx.y] : a0;
+    if (a.pv.tag == nullptr || !*a.pv.pending) return;
+    double* f = (double*)a.fin;
+    const size_t N = a.g.N;
+    for (int p = blockIdx.x; p < a.pv.np; p += gridDim.x) {
+        const PKern& k = a.pv.pk[p];
+        const int off = a.pc[p].tmpl_off + a.pc[p].n_bs, n = a.pc[p].n_is;
+        for (int e = threadIdx.x; e < n; e += blockDim.x) {
+            const int ent = a.tmpl[off + e];
+            unsigned site;
+            if (!site_fast(a.g, k.Kw, tmpl_ox(ent), tmpl_oy(ent), tmpl_oz(ent), site)) continue;
+            if (a.pv.tag[site] != ((CLS_IS << 30) | (unsigned)p)) continue;
+            const double r[3] = {(double)tmpl_ox(ent) - k.phi[0], (double)tmpl_oy(ent) - k.phi[1],
+                                 (double)tmpl_oz(ent) - k.phi[2]};
+            double u[3];
+            rigid_velocity(k, r, u);
+            feq_all_plain<L>(f[site], u, [&](auto ic, double v) { f[(size_t)decltype(ic)::value * N + site] = v; });
+        }
+    }
+}
+
+// After the sweep: the momentum transfer at the BS sites (Eqs. 5-7) with their records, and the
+// density carry of the IS sites (the sum of their populations in slot order).
+template <class L, bool B>
+__global__ void __launch_bounds__(128) k_solid_plain(const SweepArgs a0, const SweepArgs* __restrict__ cells)
+{
+    constexpr int Q = L::Q;
+    const SweepArgs& a = B ? cells[blockIdx.y] : a0;
+    if (a.pv.tag == nullptr) return;
+    double* fo = (double*)a.fout;
+    const size_t N = a.g.N;
+    for (int p = blockIdx.x; p < a.pv.np; p += gridDim.x) {
+        const PKern& k = a.pv.pk[p];
+        const int off = a.pc[p].tmpl_off, nb = a.pc[p].n_bs, n = nb + a.pc[p].n_is;
+        for (int e = threadIdx.x; e < n; e += blockDim.x) {
+            const int ent = a.tmpl[off + e];
+            unsigned site;
+            if (!site_fast(a.g, k.Kw, tmpl_ox(ent), tmpl_oy(ent), tmpl_oz(ent), site)) continue;
+            if (a.pv.tag[site] != ((tmpl_cls(ent) << 30) | (unsigned)p)) continue;
+            double f[Q];
+            sfor<0, Q>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                f[i] = fo[(size_t)i * N + site];
+            });
+            if (e >= nb) {
+                double dens = f[0];
+                sfor<1, Q>([&](auto ic) { dens += f[decltype(ic)::value]; });
+                sfor<0, Q>([&](auto ic) { fo[(size_t)decltype(ic)::value * N + site] = dens; });
+                continue;
+            }
+            const double r[3] = {(double)tmpl_ox(ent) - k.phi[0], (double)tmpl_oy(ent) - k.phi[1],
+                                 (double)tmpl_oz(ent) - k.phi[2]};
+            double rho, j[3], ubp[3], du[3];
+            rigid_velocity(k, r, ubp);
+            moments_plain<L>(f, rho, j);
+            feq_all_plain<L>(rho, ubp, [&](auto ic, double v) { fo[(size_t)decltype(ic)::value * N + site] = v; });
+#pragma unroll
+            for (int q = 0; q < 3; ++q) du[q] = ubp[q] - (q < L::D ? j[q] / rho : 0.0);
+            const double cr[3] = {r[1] * du[2] - r[2] * du[1], r[2] * du[0] - r[0] * du[2], r[0] * du[1] - r[1] * du[0]};
+            double* sc = (double*)a.bs_scratch + (size_t)site * 6;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                sc[q] = rho * du[q];
+                sc[3 + q] = rho * cr[q];
+            }
+        }
+    }
+}
+
+// Every site as fluid, sites in index order (no idle lanes at the ends of rows: an idle lane costs
+// as much FP64 issue as a busy one, and the divisions that find a site's coordinates cost none).
+// 64-thread blocks spread a small box over all SMs.
+constexpr int PLAIN_THREADS = 64;
+template <class L, bool WALLS>
+__global__ void __launch_bounds__(PLAIN_THREADS) k_sweep_plain(const SweepArgs a)
+{
+    const Geom& g = a.g;
+    const unsigned idx = blockIdx.x * PLAIN_THREADS + threadIdx.x;
+    if (idx >= g.N) return;
+    const unsigned row = idx / (unsigned)g.nx;
+    const int x = (int)(idx - row * (unsigned)g.nx);
+    const int z = (int)(row / (unsigned)g.ny);
+    const int y = (int)(row - (unsigned)z * (unsigned)g.ny);
+    const Nbr n = neighbours<WALLS>(g, x, y, z);
+    double f[L::Q];
+    pull<L, double, WALLS>((const double*)a.fin, g, n, x, y, z, idx, f);
+    sweep_site<L, double, WALLS, false>(a, x, y, z, idx, true, n, f, TAG_FLUID, 0u);
 }
 
 // In-place streaming, one phase (PHASE = SweepArgs::aa): the per-site step of k_sweep with
@@ -1218,7 +1407,8 @@ __global__ void k_is_restore(const ISFixArgs a0, const ISFixArgs* __restrict__ c
             const Nbr n = neighbours<WALLS>(g, x, y, z);
             C f[L::Q];
             pull<L, S, WALLS>((const S*)a.s.fin, g, n, x, y, z, site, f);
-            sweep_site<L, S, WALLS, true, true>(a.s, x, y, z, site, true, n, f, t, a.s.pv.ismask[site]);
+            // (FP64 storage: the input already holds the imposed values, k_impose_plain)
+            sweep_site<L, S, WALLS, Store<S>::deviation, true>(a.s, x, y, z, site, true, n, f, t, a.s.pv.ismask[site]);
         }
     }
 }
@@ -1312,6 +1502,20 @@ namespace lbmp {
 // ---- launchers --------------------------------------------------------------------------
 // Deviation storages with an even nx take the two-site kernel (a.pair_bx threads along x),
 // everything else the one-site kernel.
+// FP64 storage, pull scheme: returns the launches made.
+template <class L>
+int launch_sweep_plain(const SweepArgs& a, cudaStream_t s)
+{
+    const bool walls = a.g.wall[0] || a.g.wall[1] || a.g.wall[2];
+    const unsigned blocks = (a.g.N + PLAIN_THREADS - 1) / PLAIN_THREADS;
+    const bool part = a.pv.tag != nullptr;
+    if (part) k_impose_plain<L, false><<<std::min(a.pv.np, 65536), 128, 0, s>>>(a, nullptr);
+    if (walls) k_sweep_plain<L, true><<<blocks, PLAIN_THREADS, 0, s>>>(a);
+    else k_sweep_plain<L, false><<<blocks, PLAIN_THREADS, 0, s>>>(a);
+    if (part) k_solid_plain<L, false><<<std::min(a.pv.np, 65536), 128, 0, s>>>(a, nullptr);
+    return part ? 3 : 1;
+}
+
 template <class L, typename S, bool WALLS, bool PART>
 void launch_sweep_v(const SweepArgs& a, cudaStream_t s)
 {
@@ -1334,7 +1538,7 @@ void launch_inplace_v(const SweepArgs& a, cudaStream_t s)
 }
 
 template <class L, typename S>
-void launch_sweep_l(const SweepArgs& a, cudaStream_t s)
+int launch_sweep_l(const SweepArgs& a, cudaStream_t s)
 {
     const bool walls = a.g.wall[0] || a.g.wall[1] || a.g.wall[2];
     const bool part = a.pv.tag != nullptr;
@@ -1343,19 +1547,25 @@ void launch_sweep_l(const SweepArgs& a, cudaStream_t s)
         else if (walls) launch_inplace_v<L, S, true, false>(a, s);
         else if (part) launch_inplace_v<L, S, false, true>(a, s);
         else launch_inplace_v<L, S, false, false>(a, s);
-        return;
+        return 1;
     }
-    if (walls && part) launch_sweep_v<L, S, true, true>(a, s);
-    else if (walls) launch_sweep_v<L, S, true, false>(a, s);
-    else if (part) launch_sweep_v<L, S, false, true>(a, s);
-    else launch_sweep_v<L, S, false, false>(a, s);
+    if constexpr (!Store<S>::deviation) {
+        return launch_sweep_plain<L>(a, s);
+    } else {
+        if (walls && part) launch_sweep_v<L, S, true, true>(a, s);
+        else if (walls) launch_sweep_v<L, S, true, false>(a, s);
+        else if (part) launch_sweep_v<L, S, false, true>(a, s);
+        else launch_sweep_v<L, S, false, false>(a, s);
+        return 1;
+    }
 }
 
+// Returns the kernels launched.
 template <typename S>
-void launch_sweep(const SweepArgs& a, cudaStream_t s)
+int launch_sweep(const SweepArgs& a, cudaStream_t s)
 {
-    if (a.lattice == 0) launch_sweep_l<D2Q9, S>(a, s);
-    else launch_sweep_l<D3Q19, S>(a, s);
+    if (a.lattice == 0) return launch_sweep_l<D2Q9, S>(a, s);
+    return launch_sweep_l<D3Q19, S>(a, s);
 }
 
 template <typename S>
@@ -1486,20 +1696,30 @@ void launch_sweep_batch_v(const BatchSweepArgs& b, cudaStream_t s)
 }
 
 template <class L, typename S>
-void launch_sweep_batch_l(const BatchSweepArgs& b, cudaStream_t s)
+int launch_sweep_batch_l(const BatchSweepArgs& b, cudaStream_t s)
 {
-    if (b.walls && b.part) launch_sweep_batch_v<L, S, true, true>(b, s);
-    else if (b.walls) launch_sweep_batch_v<L, S, true, false>(b, s);
-    else if (b.part) launch_sweep_batch_v<L, S, false, true>(b, s);
-    else launch_sweep_batch_v<L, S, false, false>(b, s);
+    if constexpr (!Store<S>::deviation) {  // see k_impose_plain
+        const dim3 grid(std::max(2, 304 / b.ncells), b.ncells);
+        if (b.part) k_impose_plain<L, true><<<grid, 128, 0, s>>>(SweepArgs{}, b.cells);
+        if (b.walls) launch_sweep_batch_v<L, S, true, false>(b, s);
+        else launch_sweep_batch_v<L, S, false, false>(b, s);
+        if (b.part) k_solid_plain<L, true><<<grid, 128, 0, s>>>(SweepArgs{}, b.cells);
+        return b.part ? 3 : 1;
+    } else {
+        if (b.walls && b.part) launch_sweep_batch_v<L, S, true, true>(b, s);
+        else if (b.walls) launch_sweep_batch_v<L, S, true, false>(b, s);
+        else if (b.part) launch_sweep_batch_v<L, S, false, true>(b, s);
+        else launch_sweep_batch_v<L, S, false, false>(b, s);
+        return 1;
+    }
 }
 
 template <typename S>
-void launch_sweep_batch(const BatchSweepArgs& b, cudaStream_t s)
+int launch_sweep_batch(const BatchSweepArgs& b, cudaStream_t s)
 {
-    if (b.ntiles == 0) return;
-    if (b.lattice == 0) launch_sweep_batch_l<D2Q9, S>(b, s);
-    else launch_sweep_batch_l<D3Q19, S>(b, s);
+    if (b.ntiles == 0) return 0;
+    if (b.lattice == 0) return launch_sweep_batch_l<D2Q9, S>(b, s);
+    return launch_sweep_batch_l<D3Q19, S>(b, s);
 }
 
 template <typename S>
