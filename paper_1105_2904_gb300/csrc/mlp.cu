@@ -225,17 +225,14 @@ __global__ void k_gather(const float* __restrict__ X, const float* __restrict__ 
     }
 }
 
-// One Adam step (Kingma & Ba, 2015) of parameter i with gradient gi; returns the new value.
-__device__ __forceinline__ float adam_step(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v, long long i,
-                                           float gi, float lr, float b1, float b2, float eps, float c1, float c2)
+// One Adam step (Kingma & Ba, 2015) of parameter p with moments m, v and gradient g; c1, c2 the
+// bias corrections.
+__device__ __forceinline__ void adam_step(float& p, float& m, float& v, float g, float lr, float b1, float b2, float eps,
+                                          float c1, float c2)
 {
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    p[i] = pi;
-    return pi;
+    m = fmaf(1.f - b1, g, b1 * m);  // (explicit, so that every kernel rounds alike)
+    v = fmaf((1.f - b2) * g, g, b2 * v);
+    p = p - lr * (m / c1) / (sqrtf(v / c2) + eps);
 }
 
 // Adam on FP32 masters p with moments m, v; t_dev holds the number of
@@ -248,7 +245,11 @@ __global__ void k_adam(float* __restrict__ p, float* __restrict__ m, float* __re
     const float c1 = 1.f - powf(b1, (float)t);
     const float c2 = 1.f - powf(b2, (float)t);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float pi = adam_step(p, m, v, i, g[i], lr, b1, b2, eps, c1, c2);
+        float pi = p[i], mi = m[i], vi = v[i];
+        adam_step(pi, mi, vi, g[i], lr, b1, b2, eps, c1, c2);
+        p[i] = pi;
+        m[i] = mi;
+        v[i] = vi;
         if (p16) p16[i] = __float2bfloat16(pi);
     }
 }
@@ -261,12 +262,15 @@ __global__ void k_adam(float* __restrict__ p, float* __restrict__ m, float* __re
 // the tensor-core fragments (forward B(k, n) = W[n][k]; backward B(k = j, n = c) = W[j][c]), so a
 // lane's operand is one 8-byte load and a warp's 256 consecutive bytes, whatever the width of the
 // layer (the closure's 259 inputs leave W's rows unaligned); Adam writes its new weights there.
-// Minibatch of 128 rows: 208 us in ~20 launches -> STEPNEW us; forward pass of 200 rows 110 -> FWDNEW us.
+// Epoch of 24 minibatches of 128 rows, with the parameters read back: 4963 -> 527 us (a minibatch was
+// ~20 launches); forward pass of 200 rows 113 -> 14 us.
 
 constexpr int MAX_LAYERS = 8;
 constexpr int ROWS = 16;             // rows per block: one m16n8k16 tile
 constexpr int ROWS_THREADS = 256;
 constexpr int UPD_THREADS = 128;
+constexpr int KCHUNK = 9;            // k-steps of weights a warp loads at once (the closure's 17 in two)
+constexpr int RCHUNK = 8;            // k-steps of rows a warp of k_update loads at once (128 rows)
 constexpr int SPLITS = 16;           // fixed-order split of the rows in the weight gradients
 // Up to here a 16-row block's pass over all weights (512 kB from L2) stays a matter of a few us.
 constexpr long long FUSED_WEIGHTS = 262144;
@@ -325,11 +329,11 @@ struct UpdateArgs {
     double loss_scale;
 };
 
-// C (16 rows of `in` times a K x N operand in fragment order) for this warp's n-tiles, two at a
-// time; put(row, column, value) for the lane's elements.
+// C (16 rows of `in` times a K x N operand in fragment order, plus the bias if given) for this
+// warp's n-tiles, two at a time; put(row, column, value) for the lane's elements.
 template <class PUT>
 __device__ __forceinline__ void rows_gemm(const __nv_bfloat16* __restrict__ in, int ld, int K, int N,
-                                          const __nv_bfloat16* __restrict__ frag, PUT&& put)
+                                          const __nv_bfloat16* __restrict__ frag, const float* __restrict__ bias, PUT&& put)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gq = lane >> 2, tq = lane & 3;
@@ -338,21 +342,38 @@ __device__ __forceinline__ void rows_gemm(const __nv_bfloat16* __restrict__ in, 
         const bool two = nt + 1 < NT;
         const uint2* b0p = reinterpret_cast<const uint2*>(frag) + (long long)nt * KS * 32 + lane;
         const uint2* b1p = two ? b0p + (long long)KS * 32 : b0p;
-        float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 9
-        for (int ks = 0; ks < KS; ++ks) {
-            const uint2 v0 = b0p[ks * 32], v1 = b1p[ks * 32];
-            const __nv_bfloat16* ap = in + gq * ld + ks * 16 + 2 * tq;
-            const uint32_t a[4] = {ld_pair(ap), ld_pair(ap + 8 * ld), ld_pair(ap + 8), ld_pair(ap + 8 * ld + 8)};
-            const uint32_t b0[2] = {v0.x, v0.y}, b1[2] = {v1.x, v1.y};
-            mma_bf16(c0, a, b0);
-            mma_bf16(c1, a, b1);
+        float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f}, bs[2][2] = {};
+        if (bias) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int col = nt * 8 + 8 * (q >> 1) + 2 * tq + (q & 1);
+                if (col < N) bs[q >> 1][q & 1] = bias[col];
+            }
+        }
+        for (int k0 = 0; k0 < KS; k0 += KCHUNK) {
+            // the chunk's operands first, all in flight together
+            uint2 v0[KCHUNK], v1[KCHUNK];
+#pragma unroll
+            for (int j = 0; j < KCHUNK; ++j) {
+                const bool in_k = k0 + j < KS;
+                v0[j] = in_k ? b0p[(k0 + j) * 32] : make_uint2(0u, 0u);
+                v1[j] = in_k ? b1p[(k0 + j) * 32] : make_uint2(0u, 0u);
+            }
+#pragma unroll
+            for (int j = 0; j < KCHUNK; ++j) {
+                if (k0 + j >= KS) break;
+                const __nv_bfloat16* ap = in + gq * ld + (k0 + j) * 16 + 2 * tq;
+                const uint32_t a[4] = {ld_pair(ap), ld_pair(ap + 8 * ld), ld_pair(ap + 8), ld_pair(ap + 8 * ld + 8)};
+                const uint32_t b0[2] = {v0[j].x, v0[j].y}, b1[2] = {v1[j].x, v1[j].y};
+                mma_bf16(c0, a, b0);
+                mma_bf16(c1, a, b1);
+            }
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int row = gq + (q >= 2 ? 8 : 0), col = nt * 8 + 2 * tq + (q & 1);
-            if (col < N) put(row, col, c0[q]);
-            if (two && col + 8 < N) put(row, col + 8, c1[q]);
+            if (col < N) put(row, col, bias ? c0[q] + bs[0][q & 1] : c0[q]);
+            if (two && col + 8 < N) put(row, col + 8, bias ? c1[q] + bs[1][q & 1] : c1[q]);
         }
     }
 }
@@ -385,17 +406,29 @@ __global__ void __launch_bounds__(ROWS_THREADS) k_rows(const RowsArgs a)
             d[l] = sm + total;
             total += ROWS * tile_ld(n.size[l]);
         }
+    float* tgt = reinterpret_cast<float*>(sm + total);  // targets [ROWS][O]
     // padding rows and columns are zero
     for (int e = threadIdx.x; e < total / 8; e += ROWS_THREADS) reinterpret_cast<uint4*>(sm)[e] = make_uint4(0, 0, 0, 0);
     __syncthreads();
     // the minibatch's rows; nothing here depends on the kernel before
-    for (int e = threadIdx.x; e < ROWS * K0; e += ROWS_THREADS) {
-        const int r = e / K0, c = e - r * K0;
-        if (row0 + r >= a.rows) break;
+    // (a warp takes two rows, eight columns of each lane in flight)
+    for (int r = threadIdx.x >> 5; r < ROWS && row0 + r < a.rows; r += ROWS_THREADS / 32) {
         const long long src = a.idx ? a.idx[row0 + r] : row0 + r;
-        float v = a.X[src * K0 + c];
-        if (n.shift) v = (v - n.shift[c]) * n.scale[c];
-        h[0][r * tile_ld(K0) + c] = __float2bfloat16(v);
+        const float* x = a.X + src * K0;
+        if (train)
+            for (int c = threadIdx.x & 31; c < O; c += 32) tgt[r * O + c] = a.T[src * O + c];
+        for (int c0 = threadIdx.x & 31; c0 < K0; c0 += 8 * 32) {
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = c0 + 32 * j < K0 ? x[c0 + 32 * j] : 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int c = c0 + 32 * j;
+                if (c >= K0) continue;
+                if (n.shift) v[j] = (v[j] - n.shift[c]) * n.scale[c];
+                h[0][r * tile_ld(K0) + c] = __float2bfloat16(v[j]);
+            }
+        }
     }
     wait_for_previous_kernel();
     let_next_kernel_start();
@@ -407,20 +440,17 @@ __global__ void __launch_bounds__(ROWS_THREADS) k_rows(const RowsArgs a)
         if (l + 1 < L) {
             __nv_bfloat16* out = h[l + 1];
             const int ldo = tile_ld(N);
-            rows_gemm(h[l], tile_ld(K), K, N, n.wf + n.wf_off[l], [&](int r, int c, float v) {
-                out[r * ldo + c] = __float2bfloat16(fmaxf(v + bias[c], 0.f));
-            });
+            rows_gemm(h[l], tile_ld(K), K, N, n.wf + n.wf_off[l], bias,
+                      [&](int r, int c, float v) { out[r * ldo + c] = __float2bfloat16(fmaxf(v, 0.f)); });
         } else {
-            rows_gemm(h[l], tile_ld(K), K, N, n.wf + n.wf_off[l], [&](int r, int c, float v) {
+            rows_gemm(h[l], tile_ld(K), K, N, n.wf + n.wf_off[l], bias, [&](int r, int c, float y) {
                 if (row0 + r >= a.rows) return;
-                const float y = v + bias[c];
                 if (!train) {
                     a.y[(long long)(row0 + r) * O + c] = y;
                     return;
                 }
                 // mean-squared error: d = 2 (y - t) / (rows O)
-                const long long src = a.idx ? a.idx[row0 + r] : row0 + r;
-                const float res = y - a.T[src * O + c];
+                const float res = y - tgt[r * O + c];
                 n.r2[(long long)(row0 + r) * O + c] = res * res;
                 d[L][r * tile_ld(O) + c] = __float2bfloat16(2.f * res * a.grad_scale);
             });
@@ -431,7 +461,7 @@ __global__ void __launch_bounds__(ROWS_THREADS) k_rows(const RowsArgs a)
     // d_l = (d_{l+1} W_l) relu'(h_l)
     for (int l = L - 1; l >= 1; --l) {
         const int K = n.size[l], N = n.size[l + 1], ldk = tile_ld(K);
-        rows_gemm(d[l + 1], tile_ld(N), N, K, n.wb + n.wb_off[l], [&](int r, int c, float v) {
+        rows_gemm(d[l + 1], tile_ld(N), N, K, n.wb + n.wb_off[l], nullptr, [&](int r, int c, float v) {
             const bool on = __bfloat162float(h[l][r * ldk + c]) > 0.f;
             d[l][r * ldk + c] = __float2bfloat16(on ? v : 0.f);
         });
@@ -499,28 +529,61 @@ __global__ void __launch_bounds__(UPD_THREADS) k_update(const UpdateArgs a)
         const __nv_bfloat16* d1 = d0 + 8LL * n.ld;
         const __nv_bfloat16* hb = n.hT[l] + (long long)(k0 + gq) * n.ld + 2 * tq;
         const bool ok0 = n0 + gq < N, ok1 = n0 + gq + 8 < N, okb = k0 + gq < K;
-        float s[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int z = 0; z * per < rows16; ++z) {
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
-            const int end = min(rows16, (z + 1) * per);
-#pragma unroll 4
-            for (int r = z * per; r < end; r += 16) {
-                const uint32_t A[4] = {ok0 ? ld_pair(d0 + r) : 0u, ok1 ? ld_pair(d1 + r) : 0u, ok0 ? ld_pair(d0 + r + 8) : 0u,
-                                       ok1 ? ld_pair(d1 + r + 8) : 0u};
-                const uint32_t B[2] = {okb ? ld_pair(hb + r) : 0u, okb ? ld_pair(hb + r + 8) : 0u};
-                mma_bf16(c, A, B);
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) s[q] += c[q];
-        }
+        // this lane's parameters, loaded beside the operands
+        long long at[4];
+        float pv[4], mv[4], vv[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int nn = n0 + gq + (q >= 2 ? 8 : 0), k = k0 + 2 * tq + (q & 1);
-            if (nn >= N || k >= K) continue;
-            const long long i = n.w_off[l] + (long long)nn * K + k;
-            a.g[i] = s[q];
+            at[q] = nn < N && k < K ? n.w_off[l] + (long long)nn * K + k : -1;
+            if (a.t && at[q] >= 0) {
+                pv[q] = a.p[at[q]];
+                mv[q] = a.m[at[q]];
+                vv[q] = a.v[at[q]];
+            }
+        }
+        float s[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
+        int next = per;  // first row of the next range
+        for (int r0 = 0; r0 < rows16; r0 += 16 * RCHUNK) {
+            uint32_t A[RCHUNK][4], B[RCHUNK][2];
+#pragma unroll
+            for (int j = 0; j < RCHUNK; ++j) {
+                const int r = r0 + 16 * j;
+                const bool in = r < rows16;
+                A[j][0] = in && ok0 ? ld_pair(d0 + r) : 0u;
+                A[j][1] = in && ok1 ? ld_pair(d1 + r) : 0u;
+                A[j][2] = in && ok0 ? ld_pair(d0 + r + 8) : 0u;
+                A[j][3] = in && ok1 ? ld_pair(d1 + r + 8) : 0u;
+                B[j][0] = in && okb ? ld_pair(hb + r) : 0u;
+                B[j][1] = in && okb ? ld_pair(hb + r + 8) : 0u;
+            }
+#pragma unroll
+            for (int j = 0; j < RCHUNK; ++j) {
+                const int r = r0 + 16 * j;
+                if (r >= rows16) break;
+                if (r == next) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        s[q] += c[q];
+                        c[q] = 0.f;
+                    }
+                    next += per;
+                }
+                mma_bf16(c, A[j], B[j]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (at[q] < 0) continue;
+            s[q] += c[q];
+            a.g[at[q]] = s[q];
             if (!a.t) continue;
-            const __nv_bfloat16 w = __float2bfloat16(adam_step(a.p, a.m, a.v, i, s[q], a.lr, a.b1, a.b2, a.eps, c1, c2));
+            adam_step(pv[q], mv[q], vv[q], s[q], a.lr, a.b1, a.b2, a.eps, c1, c2);
+            a.p[at[q]] = pv[q];
+            a.m[at[q]] = mv[q];
+            a.v[at[q]] = vv[q];
+            const __nv_bfloat16 w = __float2bfloat16(pv[q]);
+            const int nn = n0 + gq + (q >= 2 ? 8 : 0), k = k0 + 2 * tq + (q & 1);
             n.wf[n.wf_off[l] + frag_pos(k, nn, K)] = w;
             if (l > 0) n.wb[n.wb_off[l] + frag_pos(nn, k, N)] = w;
         }
@@ -535,15 +598,16 @@ __global__ void __launch_bounds__(UPD_THREADS) k_update(const UpdateArgs a)
         const __nv_bfloat16* dr = n.dT[l] + (long long)task * n.ld;
         float x[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            x[j] = 0.f;
-            for (int r = lane + 32 * j; r < a.rows; r += 256) x[j] += __bfloat162float(dr[r]);
-        }
+        for (int j = 0; j < 8; ++j) x[j] = lane + 32 * j < a.rows ? __bfloat162float(dr[lane + 32 * j]) : 0.f;
+        for (int r0 = 256; r0 < a.rows; r0 += 256)
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (r0 + lane + 32 * j < a.rows) x[j] += __bfloat162float(dr[r0 + lane + 32 * j]);
         const float s = tree256(x);
         if (lane == 0) {
             const long long i = n.b_off[l] + task;
             a.g[i] = s;
-            if (a.t) adam_step(a.p, a.m, a.v, i, s, a.lr, a.b1, a.b2, a.eps, c1, c2);
+            if (a.t) adam_step(a.p[i], a.m[i], a.v[i], s, a.lr, a.b1, a.b2, a.eps, c1, c2);
         }
         return;
     }
@@ -772,7 +836,7 @@ size_t rows_smem(const lbm_mlp* net, bool train)
     for (int l = 0; l < net->L; ++l) e += (size_t)ROWS * tile_ld(net->sizes[(size_t)l]);
     if (train)
         for (int l = 1; l <= net->L; ++l) e += (size_t)ROWS * tile_ld(net->sizes[(size_t)l]);
-    return e * sizeof(__nv_bfloat16);
+    return e * sizeof(__nv_bfloat16) + (train ? sizeof(float) * ROWS * (size_t)net->sizes[(size_t)net->L] : 0);
 }
 
 NetArgs net_args(const lbm_mlp* net)
@@ -834,9 +898,9 @@ void fused_rows(lbm_mlp* net, const float* x, const float* t, const int* idx, in
     launch(k_rows, (rows + ROWS - 1) / ROWS, ROWS_THREADS, rows_smem(net, t != nullptr), overlap, net->stream, a);
 }
 
-// The gradients of the rows of the last fused_rows, the loss into loss_dev[slot], and with lr > 0
+// The gradients of the rows of the last fused_rows, the loss into loss_dev[slot], and with `step`
 // the Adam step.
-void fused_update(lbm_mlp* net, int rows, int slot, float lr, float b1, float b2, float eps)
+void fused_update(lbm_mlp* net, int rows, int slot, bool step, float lr, float b1, float b2, float eps)
 {
     UpdateArgs a{};
     a.n = net_args(net);
@@ -845,7 +909,7 @@ void fused_update(lbm_mlp* net, int rows, int slot, float lr, float b1, float b2
     a.m = net->m;
     a.v = net->v;
     a.g = net->g;
-    a.t = lr > 0.f ? net->t : nullptr;
+    a.t = step ? net->t : nullptr;
     a.lr = lr;
     a.b1 = b1;
     a.b2 = b2;
@@ -1022,7 +1086,14 @@ lbm_status lbm_mlp_forward(lbm_mlp* net, const float* x, int rows, float* y)
     if (!net || !x || !y || rows < 0) return LBM_E_INVALID;
     if (rows == 0) return LBM_OK;
     if (net->fused) {
-        fused_rows(net, x, nullptr, nullptr, rows, y, false, false);
+        const size_t nx = (size_t)rows * net->sizes[0], ny = (size_t)rows * net->sizes[(size_t)net->L];
+        const bool alias = (uintptr_t)y < (uintptr_t)(x + nx) && (uintptr_t)x < (uintptr_t)(y + ny);
+        if (alias) {  // blocks read their rows while others write theirs
+            lbm_status s = ensure_rows(net, rows);
+            if (s != LBM_OK) return s;
+        }
+        fused_rows(net, x, nullptr, nullptr, rows, alias ? net->r2 : y, false, false);
+        if (alias) MK(cudaMemcpyAsync(y, net->r2, sizeof(float) * ny, cudaMemcpyDeviceToDevice, net->stream));
         MK(cudaGetLastError());
         return LBM_OK;
     }
@@ -1047,7 +1118,7 @@ lbm_status lbm_mlp_loss_grad(lbm_mlp* net, const float* x, const float* t, int r
     MK(cudaMemsetAsync(net->loss_dev, 0, sizeof(double), net->stream));
     if (net->fused) {
         fused_rows(net, x, t, nullptr, rows, nullptr, false, false);
-        fused_update(net, rows, 0, 0.f, 0.f, 0.f, 0.f);
+        fused_update(net, rows, 0, false, 0.f, 0.f, 0.f, 0.f);
     } else {
         k_gather<<<blocks_for((long long)rows * (K + O)), 256, 0, net->stream>>>(x, t, nullptr, rows, K, O, net->in_shift,
                                                                                    net->in_scale, net->xb, net->tb);
@@ -1096,7 +1167,7 @@ lbm_status lbm_mlp_train(lbm_mlp* net, const float* x, const float* t, int n, in
             if (net->fused) {
                 // (the first minibatch follows the copy of the permutation, the others k_update)
                 fused_rows(net, x, t, net->idx + (size_t)bi * batch, batch, nullptr, true, bi > 0);
-                fused_update(net, batch, e, (float)lr, 0.9f, 0.999f, 1e-8f);
+                fused_update(net, batch, e, true, (float)lr, 0.9f, 0.999f, 1e-8f);
                 continue;
             }
             k_gather<<<blocks_for((long long)batch * (K + O)), 256, 0, net->stream>>>(x, t, net->idx + (size_t)bi * batch,
