@@ -273,6 +273,20 @@ ISFixArgs is_fix_args(lbm_ctx* ctx, int c)
     return s;
 }
 
+RemarkArgs remark_args(lbm_ctx* ctx, int c)
+{
+    RemarkArgs r{};
+    if (ctx->np > 0) {
+        r.f = is_fix_args(ctx, c);
+        if (ctx->inplace) r.f.dens = ctx->is_rho[1 - c];
+        r.p = particle_args(ctx);
+        r.m = mask_args(ctx, true);
+    }
+    r.wv = ctx->moving_walls ? ctx->wv : nullptr;
+    r.p_pending = ctx->pending;
+    return r;
+}
+
 // One time step on ctx->stream, reading buffer c and writing buffer 1 - c. With ev != nullptr
 // CUDA events are recorded before the sweep, after it, and after the particle phase.
 int enqueue_step(lbm_ctx* ctx, int c, cudaEvent_t* ev = nullptr)
@@ -286,11 +300,18 @@ int enqueue_step(lbm_ctx* ctx, int c, cudaEvent_t* ev = nullptr)
     }
     if (ev) cudaEventRecord(ev[1], ctx->stream);
     NvtxRange rp("lbm particle phase");
+    bool walls_advanced = false;
     if (ctx->np > 0) {
         const ParticleArgs pa = particle_args(ctx);
         const ISFixArgs fa = is_fix_args(ctx, c);
+        PhaseShape sh = phase_shape(pa);
+        sh.max_entries = (long long)ctx->h_tmpl.size();
         launches += launch_particle_phase_a(pa, ctx->stream);
-        if (ctx->inplace) {
+        if (few_entries(sh)) {
+            ctx->kt->remark(ctx->lattice, remark_args(ctx, c), nullptr, 1, ctx->stream);
+            launches += 1;
+            walls_advanced = ctx->moving_walls;
+        } else if (ctx->inplace) {
             // in-place streaming: the IS sites kept their populations; only the sites that
             // became IS need their density in the array the next sweep reads
             launches += launch_particle_phase_b(pa, ctx->stream);
@@ -307,7 +328,7 @@ int enqueue_step(lbm_ctx* ctx, int c, cudaEvent_t* ev = nullptr)
             launches += 4;
         }
     }
-    if (ctx->moving_walls) {
+    if (ctx->moving_walls && !walls_advanced) {
         launch_wall_advance(ctx->wv, ctx->pending, ctx->stream);
         launches += 1;
     }

@@ -33,6 +33,7 @@ struct lbm_batch {
     ISFixArgs* d_isfix[2] = {nullptr, nullptr};
     ParticleArgs* d_part = nullptr;
     MaskArgs* d_mask = nullptr;
+    RemarkArgs* d_remark[2] = {nullptr, nullptr};  // few_entries(shape): in the place of d_isfix, d_mask
     int4* d_table = nullptr;
     int ntiles = 0;
     PhaseShape shape{};
@@ -94,6 +95,7 @@ void release_device(lbm_batch* b)
     b->d_isfix[0] = b->d_isfix[1] = nullptr;
     b->d_part = nullptr;
     b->d_mask = nullptr;
+    b->d_remark[0] = b->d_remark[1] = nullptr;
     b->d_table = nullptr;
     b->built = false;
 }
@@ -129,6 +131,11 @@ int enqueue_batch_step(lbm_batch* b, int c, cudaEvent_t* ev = nullptr)
     if (b->any_part) {
         const int nc = (int)b->cells.size();
         launches += launch_particle_phase_batch_a(b->d_part, b->shape, b->stream);
+        if (few_entries(b->shape)) {
+            b->kt->remark(b->lattice, RemarkArgs{}, b->d_remark[c], nc, b->stream);
+            if (ev) cudaEventRecord(ev[2], b->stream);
+            return launches + 1;
+        }
         b->kt->is_save_batch(b->lattice, b->d_isfix[c], nc, b->stream);
         launches += launch_particle_phase_batch_b(b->d_part, b->shape, b->stream);
         b->kt->is_fix_batch(b->lattice, b->d_isfix[c], nc, b->stream);
@@ -188,6 +195,7 @@ lbm_status build(lbm_batch* b)
         b->shape.max_np = std::max(b->shape.max_np, ctx->np);
         if (ctx->np > 0) b->shape.max_cells = std::max(b->shape.max_cells, ctx->cg.total);
         max_pairs = std::max(max_pairs, (long long)ctx->np * (ctx->np - 1) / 2);
+        b->shape.max_entries = std::max(b->shape.max_entries, (long long)ctx->h_tmpl.size());
     }
     // Each cell's resolve buffer holds all its possible pairs (up to the single-context cap).
     int cap = 32;
@@ -200,8 +208,10 @@ lbm_status build(lbm_batch* b)
     std::vector<ISFixArgs> st[2];
     std::vector<ParticleArgs> pa;
     std::vector<MaskArgs> ma;
+    std::vector<RemarkArgs> ra[2];
     for (int i = 0; i < nc; ++i) {
         lbm_ctx* ctx = b->cells[(size_t)i];
+        for (int c = 0; c < 2; ++c) ra[c].push_back(remark_args(ctx, c));
         for (int c = 0; c < 2; ++c) {
             sw[c].push_back(sweep_args(ctx, c));
             st[c].push_back(ctx->np > 0 ? is_fix_args(ctx, c) : ISFixArgs{});
@@ -210,6 +220,7 @@ lbm_status build(lbm_batch* b)
             ParticleArgs p = particle_args(ctx);
             p.pair_cap = b->shape.pair_cap;
             pa.push_back(p);
+            for (int c = 0; c < 2; ++c) ra[c].back().p.pair_cap = p.pair_cap;
             ma.push_back(mask_args(ctx, true));
         } else {
             pa.push_back(ParticleArgs{});
@@ -228,12 +239,14 @@ lbm_status build(lbm_batch* b)
     std::vector<int4> table((size_t)nt);
     lbm_schedule_tiles(nc, dims.data(), b->tile_w.data(), b->order, (int*)table.data());
     b->ntiles = (int)nt;
+    const bool few = few_entries(b->shape);
     for (int c = 0; c < 2; ++c) {
         BS(upload(b, &b->d_sweep[c], sw[c]));
-        BS(upload(b, &b->d_isfix[c], st[c]));
+        if (few) BS(upload(b, &b->d_remark[c], ra[c]));
+        else BS(upload(b, &b->d_isfix[c], st[c]));
     }
     BS(upload(b, &b->d_part, pa));
-    BS(upload(b, &b->d_mask, ma));
+    if (!few) BS(upload(b, &b->d_mask, ma));
     BS(upload(b, &b->d_table, table));
     for (int c = 0; c < 2; ++c) {
         BS(capture(b, c, 1, &b->g1[c]));

@@ -174,6 +174,7 @@ MaskArgs mask_args(lbm_ctx* ctx, bool restamp_list);
 PartView part_view(lbm_ctx* ctx);
 SweepArgs sweep_args(lbm_ctx* ctx, int c);
 ISFixArgs is_fix_args(lbm_ctx* ctx, int c);
+RemarkArgs remark_args(lbm_ctx* ctx, int c);
 
 }  // namespace host
 }  // namespace lbmp

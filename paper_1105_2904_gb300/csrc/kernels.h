@@ -127,6 +127,8 @@ struct FeatureArgs {
     float* out;                // [np][n_side^3][4]
 };
 
+struct RemarkArgs;
+
 struct KernelTable {
     int (*sweep)(const SweepArgs&, cudaStream_t);  // returns the kernels launched
     void (*update_masks)(const MaskArgs&, cudaStream_t);
@@ -146,6 +148,9 @@ struct KernelTable {
     // (ISFixArgs.dens = the density array the next sweep reads; s.aa = the layout the sweep
     // left: 1 after a neighbour phase, 2 after a local phase).
     void (*inplace_fix)(const ISFixArgs&, cudaStream_t);
+    // The IS bookkeeping, the owner-map update and the masks in one launch (few_entries); cells:
+    // per-cell arguments on the device, or null.
+    void (*remark)(int lattice, const RemarkArgs&, const RemarkArgs* cells, int ncells, cudaStream_t);
     int elem_bytes;
     int compute_bytes;
 };
@@ -210,6 +215,32 @@ int launch_particle_phase_b(const ParticleArgs& a, cudaStream_t s);
 // Stamps every particle's site set into a cleared owner map (after lbm_add_particles).
 void launch_stamp_all(const ParticleArgs& a, cudaStream_t s);
 
+// Arguments of k_remark (sweep.cuh): the re-marking of one step in one launch.
+constexpr int REMARK_CLUSTER = 8, REMARK_CLUSTER_BATCH = 4;
+constexpr long long REMARK_ENTRIES = 262144;
+struct RemarkArgs {
+    ISFixArgs f;               // (f.dens: in-place streaming's density array there)
+    ParticleArgs p;
+    MaskArgs m;
+    WallVel* wv;               // moving walls: their velocities, advanced at the end; or null
+    int* p_pending;
+};
+
+// A barrier of the CS blocks of a cluster (of one block for CS = 1); what they wrote before it, to
+// global memory too, they see after it (release and acquire at cluster scope).
+#ifdef __CUDACC__
+template <int CS>
+__device__ __forceinline__ void cluster_barrier()
+{
+    if constexpr (CS > 1) {
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    } else {
+        __syncthreads();
+    }
+}
+#endif
+
 // Shape of a batched particle phase: the largest per-cell counts size the grids
 // (blockIdx.y = cell; blocks beyond a cell's own counts return at once).
 struct PhaseShape {
@@ -218,7 +249,14 @@ struct PhaseShape {
     int max_cells;    // contact-grid cells of the largest cell
     int pair_cap;     // contact-pair capacity of every cell (its resolve buffer)
     int scratch_f64;  // FP64 storage: ordered per-particle sums
+    long long max_entries;  // template entries of the cell with the most
 };
+// The shape of a single context (max_entries is the caller's to set).
+PhaseShape phase_shape(const ParticleArgs& a);
+// Few enough particles for the two-launch form of phase (a) (particles.cu), and few enough
+// template entries for k_remark in the place of what follows.
+bool few_particles(const PhaseShape& sh);
+inline bool few_entries(const PhaseShape& sh) { return few_particles(sh) && sh.max_entries <= REMARK_ENTRIES; }
 int launch_particle_phase_batch_a(const ParticleArgs* cells, const PhaseShape& sh, cudaStream_t s);
 int launch_particle_phase_batch_b(const ParticleArgs* cells, const PhaseShape& sh, cudaStream_t s);
 // After a sweep with moving walls: the current wall velocities become those of the streaming

@@ -36,6 +36,7 @@
 #include <algorithm>
 
 #include "kernels.h"
+#include "marking.cuh"
 
 namespace lbmp {
 
@@ -666,6 +667,32 @@ __device__ __forceinline__ void is_density_from_array_warp(const Geom& g, const 
     if (m & MASK_OTHER) is_density_from_array<L, C, WALLS>(g, n, x, y, z, idx, MASK_OTHER, pv, rho, f);
 }
 
+// Rebuilds the IS-source mask at the site of template entry e of particle p.
+template <class L>
+__device__ __forceinline__ void mask_entry(const MaskArgs& a, int p, int e)
+{
+    const Geom& g = a.g;
+    const int Kw[3] = {a.pk[p].Kw[0], a.pk[p].Kw[1], a.pk[p].Kw[2]};
+    const int ent = a.tmpl[a.pc[p].tmpl_off + e];
+    unsigned idx;
+    int v[3];
+    if (!site_fast_xyz(g, Kw, tmpl_ox(ent), tmpl_oy(ent), tmpl_oz(ent), idx, v)) return;
+    const unsigned owner = a.tag[idx] & PID_MASK;
+    const int x = v[0], y = v[1], z = v[2];
+    const Nbr n = neighbours<true>(g, x, y, z);
+    unsigned m = 0;
+    sfor<0, L::Q>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        int sx, sy, sz;
+        unsigned sidx;
+        bool bounce;
+        pull_source<L, i, true>(g, n, x, y, z, idx, sx, sy, sz, sidx, bounce);
+        const unsigned t = a.tag[sidx];
+        if ((t >> 30) == CLS_IS) m |= ((t & PID_MASK) == owner) ? (1u << i) : MASK_OTHER;
+    });
+    a.ismask[idx] = m;
+}
+
 // Rebuilds the IS-source masks at the sites of the listed particles (their site sets hold
 // every site whose mask can be non-zero or can have changed).
 template <class L, bool B>
@@ -674,32 +701,9 @@ __global__ void k_update_masks(const MaskArgs a0, const MaskArgs* __restrict__ c
     const MaskArgs a = pick_args<B>(a0, cells);
     if (a.np == 0 || (a.list && !a.cnt)) return;
     const int count = a.list ? a.cnt->nrestamp : a.np;
-    const Geom& g = a.g;
     for (int b = blockIdx.x; b < count; b += gridDim.x) {
         const int p = a.list ? a.list[b] : b;
-        const PConst pc = a.pc[p];
-        const int Kw[3] = {a.pk[p].Kw[0], a.pk[p].Kw[1], a.pk[p].Kw[2]};
-        for (int e = threadIdx.x; e < pc.tmpl_n; e += blockDim.x) {
-            const int ent = a.tmpl[pc.tmpl_off + e];
-            unsigned idx;
-            int v[3];
-            if (!site_fast_xyz(g, Kw, tmpl_ox(ent), tmpl_oy(ent), tmpl_oz(ent), idx, v)) continue;
-            const unsigned t0 = a.tag[idx];
-            const unsigned owner = t0 & PID_MASK;
-            const int x = v[0], y = v[1], z = v[2];
-            const Nbr n = neighbours<true>(g, x, y, z);
-            unsigned m = 0;
-            sfor<0, L::Q>([&](auto ic) {
-                constexpr int i = decltype(ic)::value;
-                int sx, sy, sz;
-                unsigned sidx;
-                bool bounce;
-                pull_source<L, i, true>(g, n, x, y, z, idx, sx, sy, sz, sidx, bounce);
-                const unsigned t = a.tag[sidx];
-                if ((t >> 30) == CLS_IS) m |= ((t & PID_MASK) == owner) ? (1u << i) : MASK_OTHER;
-            });
-            a.ismask[idx] = m;
-        }
+        for (int e = threadIdx.x; e < a.pc[p].tmpl_n; e += blockDim.x) mask_entry<L>(a, p, e);
     }
 }
 
@@ -1357,102 +1361,110 @@ __device__ __forceinline__ bool is_entry_site(const ISFixArgs& a, const int K[3]
     return site_fast(a.s.g, Kw, tmpl_ox(ent), tmpl_oy(ent), tmpl_oz(ent), site);
 }
 
+// Entry e of the visited sites of moved particle p: its IS template entries at the old anchor,
+// then at the new one.
+__device__ __forceinline__ bool visited_site(const ISFixArgs& a, int p, int e, unsigned& site)
+{
+    const int n_is = a.pc[p].n_is;
+    const bool old = e < n_is;
+    const int K[3] = {old ? a.Kold[(size_t)p * 3] : a.pk[p].K[0], old ? a.Kold[(size_t)p * 3 + 1] : a.pk[p].K[1],
+                      old ? a.Kold[(size_t)p * 3 + 2] : a.pk[p].K[2]};
+    return is_entry_site(a, K, a.pc[p].tmpl_off + a.pc[p].n_bs + e % n_is, site);
+}
+
 // (1) Before the owner map changes: the density of every visited site, read from the
 // sweep's output (one slot of a site the sweep saw as IS, else the sum of its populations in
 // slot order, the sum the sweep takes).
-template <class L, typename S, bool B>
-__global__ void k_is_density(const ISFixArgs a0, const ISFixArgs* __restrict__ cells)
+template <class L, typename S>
+__device__ __forceinline__ void is_density_entry(const ISFixArgs& a, int p, int e)
 {
     using St = Store<S>;
     using C = typename St::C;
+    const size_t N = a.s.g.N;
+    const S* fo = (const S*)a.s.fout;
+    unsigned site;
+    if (!visited_site(a, p, e, site)) return;
+    C d = (C)0;
+    if ((a.s.pv.tag[site] >> 30) == CLS_IS) {
+        d = St::load(fo[site], (C)L::w(0));
+    } else {
+        sfor<0, L::Q>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            d += St::load(fo[(size_t)i * N + site], (C)L::w(i));
+        });
+    }
+    ((C*)a.dens)[site] = d;
+}
+
+template <class L, typename S, bool B>
+__global__ void k_is_density(const ISFixArgs a0, const ISFixArgs* __restrict__ cells)
+{
     const ISFixArgs a = pick_args<B>(a0, cells);
     if (!a.cnt) return;
     const int nlist = a.cnt->nchanged;
-    const size_t N = a.s.g.N;
-    const S* fo = (const S*)a.s.fout;
-    C* dens = (C*)a.dens;
-    for (int b = blockIdx.x; b < nlist; b += gridDim.x) {
-        const int p = a.list[b];
-        const PConst pc = a.pc[p];
-        const int Ko[3] = {a.Kold[(size_t)p * 3], a.Kold[(size_t)p * 3 + 1], a.Kold[(size_t)p * 3 + 2]};
-        const int Kn[3] = {a.pk[p].K[0], a.pk[p].K[1], a.pk[p].K[2]};
-        for (int e = threadIdx.x; e < 2 * pc.n_is; e += blockDim.x) {
-            unsigned site;
-            if (!is_entry_site(a, e < pc.n_is ? Ko : Kn, pc.tmpl_off + pc.n_bs + e % pc.n_is, site)) continue;
-            C d = (C)0;
-            if ((a.s.pv.tag[site] >> 30) == CLS_IS) {
-                d = St::load(fo[site], (C)L::w(0));
-            } else {
-                sfor<0, L::Q>([&](auto ic) {
-                    constexpr int i = decltype(ic)::value;
-                    d += St::load(fo[(size_t)i * N + site], (C)L::w(i));
-                });
-            }
-            dens[site] = d;
-        }
-    }
+    for (int b = blockIdx.x; b < nlist; b += gridDim.x)
+        for (int p = a.list[b], e = threadIdx.x; e < 2 * a.pc[p].n_is; e += blockDim.x) is_density_entry<L, S>(a, p, e);
 }
 
 // (2) Still before the owner map changes: the sites the sweep saw as IS of a particle whose
 // shift changed get the populations the sweep computed for them (recomputed from the
 // sweep's input with the sweep's particle view; same code, same result bit for bit).
+template <class L, typename S, bool WALLS>
+__device__ __forceinline__ void is_restore_entry(const ISFixArgs& a, int p, int e)
+{
+    using C = typename Store<S>::C;
+    const Geom& g = a.s.g;
+    const int Ko[3] = {a.Kold[(size_t)p * 3], a.Kold[(size_t)p * 3 + 1], a.Kold[(size_t)p * 3 + 2]};
+    unsigned site;
+    if (!is_entry_site(a, Ko, a.pc[p].tmpl_off + a.pc[p].n_bs + e, site)) return;
+    const unsigned t = a.s.pv.tag[site];
+    if (t != ((CLS_IS << 30) | (unsigned)p)) return;
+    const int x = (int)(site % (unsigned)g.nx);
+    const int y = (int)((site / (unsigned)g.nx) % (unsigned)g.ny);
+    const int z = (int)(site / ((unsigned)g.nx * (unsigned)g.ny));
+    const Nbr n = neighbours<WALLS>(g, x, y, z);
+    C f[L::Q];
+    pull<L, S, WALLS>((const S*)a.s.fin, g, n, x, y, z, site, f);
+    // (FP64 storage: the input already holds the imposed values, k_impose_plain)
+    sweep_site<L, S, WALLS, Store<S>::deviation, true>(a.s, x, y, z, site, true, n, f, t, a.s.pv.ismask[site]);
+}
+
 template <class L, typename S, bool WALLS, bool B>
 __global__ void k_is_restore(const ISFixArgs a0, const ISFixArgs* __restrict__ cells)
 {
-    using C = typename Store<S>::C;
     const ISFixArgs a = pick_args<B>(a0, cells);
     if (!a.cnt) return;
     const int nlist = a.cnt->nchanged;
-    const Geom& g = a.s.g;
-    for (int b = blockIdx.x; b < nlist; b += gridDim.x) {
-        const int p = a.list[b];
-        const PConst pc = a.pc[p];
-        const int Ko[3] = {a.Kold[(size_t)p * 3], a.Kold[(size_t)p * 3 + 1], a.Kold[(size_t)p * 3 + 2]};
-        for (int e = threadIdx.x; e < pc.n_is; e += blockDim.x) {
-            unsigned site;
-            if (!is_entry_site(a, Ko, pc.tmpl_off + pc.n_bs + e, site)) continue;
-            const unsigned t = a.s.pv.tag[site];
-            if (t != ((CLS_IS << 30) | (unsigned)p)) continue;
-            const int x = (int)(site % (unsigned)g.nx);
-            const int y = (int)((site / (unsigned)g.nx) % (unsigned)g.ny);
-            const int z = (int)(site / ((unsigned)g.nx * (unsigned)g.ny));
-            const Nbr n = neighbours<WALLS>(g, x, y, z);
-            C f[L::Q];
-            pull<L, S, WALLS>((const S*)a.s.fin, g, n, x, y, z, site, f);
-            // (FP64 storage: the input already holds the imposed values, k_impose_plain)
-            sweep_site<L, S, WALLS, Store<S>::deviation, true>(a.s, x, y, z, site, true, n, f, t, a.s.pv.ismask[site]);
-        }
-    }
+    for (int b = blockIdx.x; b < nlist; b += gridDim.x)
+        for (int p = a.list[b], e = threadIdx.x; e < a.pc[p].n_is; e += blockDim.x) is_restore_entry<L, S, WALLS>(a, p, e);
 }
 
 // (3) After re-marking: every visited site that is now IS holds its density in every slot.
-template <class L, typename S, bool B>
-__global__ void k_is_fix(const ISFixArgs a0, const ISFixArgs* __restrict__ cells)
+template <class L, typename S>
+__device__ __forceinline__ void is_fix_entry(const ISFixArgs& a, int p, int e)
 {
     using St = Store<S>;
     using C = typename St::C;
+    const size_t N = a.s.g.N;
+    S* fo = (S*)a.s.fout;
+    unsigned site;
+    if (!visited_site(a, p, e, site)) return;
+    if ((a.s.pv.tag[site] >> 30) != CLS_IS) return;
+    const C d = ((const C*)a.dens)[site];
+    sfor<0, L::Q>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        fo[(size_t)i * N + site] = St::save(d, (C)L::w(i));
+    });
+}
+
+template <class L, typename S, bool B>
+__global__ void k_is_fix(const ISFixArgs a0, const ISFixArgs* __restrict__ cells)
+{
     const ISFixArgs a = pick_args<B>(a0, cells);
     if (!a.cnt) return;
     const int nlist = a.cnt->nchanged;
-    const size_t N = a.s.g.N;
-    S* fo = (S*)a.s.fout;
-    const C* dens = (const C*)a.dens;
-    for (int b = blockIdx.x; b < nlist; b += gridDim.x) {
-        const int p = a.list[b];
-        const PConst pc = a.pc[p];
-        const int Ko[3] = {a.Kold[(size_t)p * 3], a.Kold[(size_t)p * 3 + 1], a.Kold[(size_t)p * 3 + 2]};
-        const int Kn[3] = {a.pk[p].K[0], a.pk[p].K[1], a.pk[p].K[2]};
-        for (int e = threadIdx.x; e < 2 * pc.n_is; e += blockDim.x) {
-            unsigned site;
-            if (!is_entry_site(a, e < pc.n_is ? Ko : Kn, pc.tmpl_off + pc.n_bs + e % pc.n_is, site)) continue;
-            if ((a.s.pv.tag[site] >> 30) != CLS_IS) continue;
-            const C d = dens[site];
-            sfor<0, L::Q>([&](auto ic) {
-                constexpr int i = decltype(ic)::value;
-                fo[(size_t)i * N + site] = St::save(d, (C)L::w(i));
-            });
-        }
-    }
+    for (int b = blockIdx.x; b < nlist; b += gridDim.x)
+        for (int p = a.list[b], e = threadIdx.x; e < 2 * a.pc[p].n_is; e += blockDim.x) is_fix_entry<L, S>(a, p, e);
 }
 
 // In-place streaming, after re-marking: every visited site that is now IS gets its density
@@ -1460,48 +1472,103 @@ __global__ void k_is_fix(const ISFixArgs a0, const ISFixArgs* __restrict__ cells
 // (the sum the sweep takes), found where the sweep's phase left them (s.aa: 2 = slot i of x;
 // 1 = slot opp(i) of x + c_i, or slot i of x where x + c_i lies beyond a wall).
 template <class L, typename S, bool WALLS>
-__global__ void k_inplace_fix(const ISFixArgs a)
+__device__ __forceinline__ void inplace_fix_entry(const ISFixArgs& a, int p, int e)
 {
     using St = Store<S>;
     using C = typename St::C;
-    if (!a.cnt) return;
-    const int nlist = a.cnt->nchanged;
     const Geom& g = a.s.g;
     const size_t N = g.N;
     const S* fo = (const S*)a.s.fout;
-    C* dens = (C*)a.dens;
-    for (int b = blockIdx.x; b < nlist; b += gridDim.x) {
-        const int p = a.list[b];
-        const PConst pc = a.pc[p];
-        const int Ko[3] = {a.Kold[(size_t)p * 3], a.Kold[(size_t)p * 3 + 1], a.Kold[(size_t)p * 3 + 2]};
-        const int Kn[3] = {a.pk[p].K[0], a.pk[p].K[1], a.pk[p].K[2]};
-        for (int e = threadIdx.x; e < 2 * pc.n_is; e += blockDim.x) {
-            unsigned site;
-            if (!is_entry_site(a, e < pc.n_is ? Ko : Kn, pc.tmpl_off + pc.n_bs + e % pc.n_is, site)) continue;
-            if ((a.s.pv.tag[site] >> 30) != CLS_IS) continue;
-            C d = (C)0;
-            if (a.s.aa == 2) {
-                sfor<0, L::Q>([&](auto ic) {
-                    constexpr int i = decltype(ic)::value;
-                    d += St::load(fo[(size_t)i * N + site], (C)L::w(i));
-                });
-            } else {
-                const int x = (int)(site % (unsigned)g.nx);
-                const int y = (int)((site / (unsigned)g.nx) % (unsigned)g.ny);
-                const int z = (int)(site / ((unsigned)g.nx * (unsigned)g.ny));
-                const Nbr n = neighbours<WALLS>(g, x, y, z);
-                sfor<0, L::Q>([&](auto ic) {
-                    constexpr int i = decltype(ic)::value;
-                    int tx, ty, tz;
-                    unsigned tidx;
-                    bool beyond;
-                    pull_source<L, L::opp(i), WALLS>(g, n, x, y, z, site, tx, ty, tz, tidx, beyond);
-                    const size_t at = beyond ? (size_t)i * N + site : (size_t)L::opp(i) * N + tidx;
-                    d += St::load(fo[at], (C)L::w(i));
-                });
-            }
-            dens[site] = d;
+    unsigned site;
+    if (!visited_site(a, p, e, site)) return;
+    if ((a.s.pv.tag[site] >> 30) != CLS_IS) return;
+    C d = (C)0;
+    if (a.s.aa == 2) {
+        sfor<0, L::Q>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            d += St::load(fo[(size_t)i * N + site], (C)L::w(i));
+        });
+    } else {
+        const int x = (int)(site % (unsigned)g.nx);
+        const int y = (int)((site / (unsigned)g.nx) % (unsigned)g.ny);
+        const int z = (int)(site / ((unsigned)g.nx * (unsigned)g.ny));
+        const Nbr n = neighbours<WALLS>(g, x, y, z);
+        sfor<0, L::Q>([&](auto ic) {
+            constexpr int i = decltype(ic)::value;
+            int tx, ty, tz;
+            unsigned tidx;
+            bool beyond;
+            pull_source<L, L::opp(i), WALLS>(g, n, x, y, z, site, tx, ty, tz, tidx, beyond);
+            const size_t at = beyond ? (size_t)i * N + site : (size_t)L::opp(i) * N + tidx;
+            d += St::load(fo[at], (C)L::w(i));
+        });
+    }
+    ((C*)a.dens)[site] = d;
+}
+
+template <class L, typename S, bool WALLS>
+__global__ void k_inplace_fix(const ISFixArgs a)
+{
+    if (!a.cnt) return;
+    const int nlist = a.cnt->nchanged;
+    for (int b = blockIdx.x; b < nlist; b += gridDim.x)
+        for (int p = a.list[b], e = threadIdx.x; e < 2 * a.pc[p].n_is; e += blockDim.x) inplace_fix_entry<L, S, WALLS>(a, p, e);
+}
+
+// ---- few template entries: the whole re-marking in one launch ---------------------------------
+// The kernels above and the owner-map update between them are six launches of 2.5 us that find
+// nothing to do in most steps of a small suspension (a sphere at u = 1e-3 crosses a site boundary
+// once in some 300 steps). Here they are one: a cluster of 8 blocks returns at once when no shift
+// changed, and otherwise spreads each moved particle's entries over its 4096 threads with a
+// cluster barrier where the launches had a boundary. Above REMARK_ENTRIES template entries in all,
+// a fast suspension could change more of them in a step than a cluster gets through in the time
+// the launches take, so larger ones keep the launches.
+constexpr int REMARK_T = 512;
+template <class L, typename S, bool WALLS, bool B, bool INPLACE>
+__global__ void __launch_bounds__(REMARK_T) k_remark(const RemarkArgs a0, const RemarkArgs* __restrict__ cells)
+{
+    constexpr int CS = B ? REMARK_CLUSTER_BATCH : REMARK_CLUSTER;
+    const RemarkArgs& a = B ? cells[blockIdx.y] : a0;
+    const int g = (int)blockIdx.x * REMARK_T + (int)threadIdx.x;
+    constexpr int G = CS * REMARK_T;
+    // f(p, e) for the first count(p) entries of every listed particle: the cluster's threads are
+    // split into as many groups of at least 128 as there are particles
+    auto each = [&](const int* list, int n, auto count, auto f) {
+        int groups = 1;
+        while (groups * 2 <= n && groups < G / 128) groups *= 2;
+        const int size = G / groups;
+        for (int b = g / size; b < n; b += groups) {
+            const int p = list[b], m = count(p);
+            for (int e = g % size; e < m; e += size) f(p, e);
         }
+    };
+    auto visited = [&](int p) { return 2 * a.f.pc[p].n_is; };
+    auto all = [&](int p) { return a.f.pc[p].tmpl_n; };
+    const int moved = a.f.cnt ? a.f.cnt->nchanged : 0;  // (a cell of a batch may have no particles)
+    if (moved > 0) {
+        if constexpr (!INPLACE) {
+            each(a.f.list, moved, visited, [&](int p, int e) { is_density_entry<L, S>(a.f, p, e); });
+            cluster_barrier<CS>();
+            each(a.f.list, moved, [&](int p) { return a.f.pc[p].n_is; },
+                 [&](int p, int e) { is_restore_entry<L, S, WALLS>(a.f, p, e); });
+            cluster_barrier<CS>();
+        }
+        each(a.f.list, moved, all, [&](int p, int e) { clear_entry(a.p, p, OldAnchor(a.p, p), e); });
+        cluster_barrier<CS>();
+        const int restamped = a.f.cnt->nrestamp;
+        each(a.p.restamp, restamped, all, [&](int p, int e) { stamp_entry(a.p, p, e); });
+        cluster_barrier<CS>();
+        each(a.f.list, moved, visited, [&](int p, int e) {
+            if constexpr (INPLACE) inplace_fix_entry<L, S, WALLS>(a.f, p, e);
+            else is_fix_entry<L, S>(a.f, p, e);
+        });
+        each(a.p.restamp, restamped, all, [&](int p, int e) { mask_entry<L>(a.m, p, e); });
+    }
+    // the streaming of the next pull takes the current wall velocities (k_wall_advance)
+    if (a.wv && g < 18) {
+        a.wv[0].u[g / 3][g % 3] = a.wv[1].u[g / 3][g % 3];
+        a.wv[0].uf[g / 3][g % 3] = a.wv[1].uf[g / 3][g % 3];
+        if (g == 0) *a.p_pending = 1;
     }
 }
 
@@ -1670,6 +1737,47 @@ void launch_inplace_fix(const ISFixArgs& a, cudaStream_t s)
     }
 }
 
+inline void launch_cluster(const void* k, dim3 grid, int cluster, int threads, void** args, cudaStream_t s)
+{
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3((unsigned)threads);
+    c.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)cluster;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    cudaLaunchKernelExC(&c, k, args);
+}
+
+template <class L, typename S>
+void launch_remark_l(const RemarkArgs& a, const RemarkArgs* cells, int ncells, cudaStream_t s)
+{
+    RemarkArgs arg = a;
+    void* args[2] = {&arg, &cells};
+    if (cells) {
+        launch_cluster((const void*)k_remark<L, S, true, true, false>, dim3(REMARK_CLUSTER_BATCH, ncells),
+                       REMARK_CLUSTER_BATCH, REMARK_T, args, s);
+        return;
+    }
+    const bool walls = a.f.s.g.wall[0] || a.f.s.g.wall[1] || a.f.s.g.wall[2];
+    const void* k;
+    if (a.f.s.aa) k = walls ? (const void*)k_remark<L, S, true, false, true> : (const void*)k_remark<L, S, false, false, true>;
+    else k = walls ? (const void*)k_remark<L, S, true, false, false> : (const void*)k_remark<L, S, false, false, false>;
+    launch_cluster(k, dim3(REMARK_CLUSTER), REMARK_CLUSTER, REMARK_T, args, s);
+}
+
+// cells: per-cell arguments of a batch on the device (a's are not read then), or null.
+template <typename S>
+void launch_remark(int lattice, const RemarkArgs& a, const RemarkArgs* cells, int ncells, cudaStream_t s)
+{
+    if (lattice == 0) launch_remark_l<D2Q9, S>(a, cells, ncells, s);
+    else launch_remark_l<D3Q19, S>(a, cells, ncells, s);
+}
+
 template <typename S>
 void launch_update_masks(const MaskArgs& a, cudaStream_t s)
 {
@@ -1753,6 +1861,7 @@ const KernelTable* make_table()
                                   launch_update_masks_batch<S>,
                                   launch_features<S>,
                                   launch_inplace_fix<S>,
+                                  launch_remark<S>,
                                   (int)sizeof(S),
                                   (int)sizeof(typename Store<S>::C)};
     return &t;
