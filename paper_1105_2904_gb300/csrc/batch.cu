@@ -35,7 +35,8 @@ struct lbm_batch {
     MaskArgs* d_mask = nullptr;
     RemarkArgs* d_remark[2] = {nullptr, nullptr};  // few_entries(shape): in the place of d_isfix, d_mask
     int4* d_table = nullptr;
-    int ntiles = 0;
+    int ntiles = 0;             // of the schedule (lbm_schedule_tiles)
+    int launch_tiles = 0;       // of d_table (sweep_tiles)
     PhaseShape shape{};
     bool any_part = false, any_walls = false;
     std::vector<int> moving;  // cells with moving walls
@@ -121,7 +122,7 @@ int enqueue_batch_step(lbm_batch* b, int c, cudaEvent_t* ev = nullptr)
     a.cells = b->d_sweep[c];
     a.ncells = (int)b->cells.size();
     a.table = b->d_table;
-    a.ntiles = b->ntiles;
+    a.ntiles = b->launch_tiles;
     a.walls = b->any_walls ? 1 : 0;
     a.part = b->any_part ? 1 : 0;
     a.grid = b->grid;
@@ -165,6 +166,44 @@ lbm_status capture(lbm_batch* b, int c, int nsteps, cudaGraphExec_t* out)
     if (ie != cudaSuccess) return bfail(b, LBM_E_CUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ie));
     b->launches_per_step = launches;
     return LBM_OK;
+}
+
+// The tiles the sweep runs, in the schedule's order. A cell whose row tiles (of its tuned width) leave
+// more than a tenth of their lanes idle is swept in index order instead (deviation storages; 128
+// consecutive sites a tile, no lane idle; index_order has both sides measured). 64-cell ensemble,
+// least wasteful widths, FP32: sweep 1.062 -> 0.958 ms.
+std::vector<int4> sweep_tiles(const lbm_batch* b)
+{
+    const int nc = (int)b->cells.size();
+    std::vector<std::vector<int4>> per((size_t)nc);
+    for (int i = 0; i < nc; ++i) {
+        const Geom& g = b->cells[(size_t)i]->g;
+        const int dims[3] = {g.nx, g.ny, g.nz};
+        std::vector<int4>& t = per[(size_t)i];
+        t.resize((size_t)lbm_schedule_tiles(1, dims, &b->tile_w[(size_t)i], 0, nullptr));
+        if (b->precision != LBM_FP64 && 10 * (unsigned long long)g.N < 9ull * 128ull * t.size()) {
+            t.clear();
+            for (unsigned first = 0; first < g.N; first += 128u) t.push_back(make_int4(i, (int)first, -1, 0));
+        } else {
+            lbm_schedule_tiles(1, dims, &b->tile_w[(size_t)i], 0, (int*)t.data());
+            for (int4& e : t) e.x = i;
+        }
+    }
+    std::vector<int4> out;
+    if (b->order == 1) {  // one tile of each cell in turn
+        size_t longest = 0;
+        for (auto& v : per) longest = std::max(longest, v.size());
+        for (size_t j = 0; j < longest; ++j)
+            for (auto& v : per)
+                if (j < v.size()) out.push_back(v[j]);
+        return out;
+    }
+    std::vector<int> seq((size_t)nc);
+    std::iota(seq.begin(), seq.end(), 0);
+    if (b->order == 2)  // largest cell first (ties by index)
+        std::stable_sort(seq.begin(), seq.end(), [&](int x, int y) { return b->cells[(size_t)x]->g.N > b->cells[(size_t)y]->g.N; });
+    for (int i : seq) out.insert(out.end(), per[(size_t)i].begin(), per[(size_t)i].end());
+    return out;
 }
 
 // Device argument arrays, the schedule table and the step graphs.
@@ -236,9 +275,10 @@ lbm_status build(lbm_batch* b)
     const long long nt = lbm_schedule_tiles(nc, dims.data(), b->tile_w.data(), b->order, nullptr);
     if (nt < 0) return bfail(b, LBM_E_INVALID, "schedule");
     if (nt >= (1ll << 31)) return bfail(b, LBM_E_INVALID, "too many tiles");
-    std::vector<int4> table((size_t)nt);
-    lbm_schedule_tiles(nc, dims.data(), b->tile_w.data(), b->order, (int*)table.data());
+    const std::vector<int4> table = sweep_tiles(b);
+    if (table.size() >= (1ull << 31)) return bfail(b, LBM_E_INVALID, "too many tiles");
     b->ntiles = (int)nt;
+    b->launch_tiles = (int)table.size();
     const bool few = few_entries(b->shape);
     for (int c = 0; c < 2; ++c) {
         BS(upload(b, &b->d_sweep[c], sw[c]));

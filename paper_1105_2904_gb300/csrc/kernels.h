@@ -26,6 +26,7 @@ struct SweepArgs {
     float omega_f, pre_f, F_f[3];  // the same in FP32 (reduced-storage sweeps)
     int moving_walls;          // 1: wall faces may move (uw is read)
     const WallVel* uw;         // wall velocities of the streaming that the pull completes
+    int ahead;                 // k_sweep2: groups of rows to prefetch ahead (0: none)
     int pair_bx;               // deviation storage, even nx: two-site kernel with this many
                                // threads along x (16, 32, 64 or 128); 0: one-site kernel
     // In-place streaming (fin == fout, one buffer): 0 = the pull scheme above; 1 = the
@@ -103,7 +104,8 @@ struct MaskArgs {
 
 // One sweep launch over a batch of independent cells. Entry e of the schedule table is one
 // 128-thread tile of one cell: (cell, x0, y0 | log2(tile width) << 16, z); the tile covers
-// x0 .. x0 + w - 1 and y0 .. y0 + 128/w - 1 of plane z (w = 32, 64 or 128).
+// x0 .. x0 + w - 1 and y0 .. y0 + 128/w - 1 of plane z (w = 32, 64 or 128); or, with a negative third
+// entry (deviation storages), 128 sites in index order from the second entry on.
 struct BatchSweepArgs {
     int lattice;
     const SweepArgs* cells;    // device [ncells], this step's buffer parity

@@ -913,19 +913,53 @@ __device__ __forceinline__ void sweep_site(const SweepArgs& a, int x, int y, int
 }
 
 
-// Deviation storages without walls are held to nine blocks per SM (56 registers, no spills).
-template <class L, typename S, bool WALLS, bool PART>
-__global__ void __launch_bounds__(SWEEP_THREADS, (Store<S>::deviation && !WALLS) ? 9 : 1) k_sweep(const SweepArgs a)
+// The site of a thread of the one-site kernels, and whether it is the thread's to work on (a thread
+// beyond the end takes a site it never stores). Rows: 128-site tiles of one row (block x, y, z). FLAT:
+// sites in index order, which leaves no lane idle whatever the row length and costs the divisions
+// that find the coordinates.
+template <bool FLAT>
+__device__ __forceinline__ bool one_site(const Geom& g, int& x, int& y, int& z, unsigned& idx)
+{
+    if constexpr (FLAT) {
+        const unsigned at = blockIdx.x * SWEEP_THREADS + threadIdx.x;
+        idx = min(at, g.N - 1u);
+        const unsigned row = idx / (unsigned)g.nx;
+        x = (int)(idx - row * (unsigned)g.nx);
+        z = (int)(row / (unsigned)g.ny);
+        y = (int)(row - (unsigned)z * (unsigned)g.ny);
+        return at < g.N;
+    } else {
+        y = blockIdx.y;
+        z = blockIdx.z;
+        const unsigned row = ((unsigned)z * (unsigned)g.ny + (unsigned)y) * (unsigned)g.nx;
+        const int xr = blockIdx.x * SWEEP_THREADS + threadIdx.x;
+        x = min(xr, g.nx - 1);
+        idx = row + (unsigned)x;
+        return xr < g.nx;
+    }
+}
+
+// Index order pays where row tiles leave more than a tenth of their lanes idle. Sweep ms, FP32, rows
+// and index order: 161 x 93 x 117 walled (63 % of the lanes busy) 0.109 and 0.074; in-place
+// 200 x 210 x 220 (78 %) 0.372 and 0.343; 255 x 254 x 253 (99.6 %) 0.513 and 0.533; in-place
+// 384^3 (100 %) 1.949 and 2.045.
+inline bool index_order(const Geom& g)
+{
+    const int lanes = (g.nx + SWEEP_THREADS - 1) / SWEEP_THREADS * SWEEP_THREADS;
+    return 10 * (long long)g.nx < 9 * (long long)lanes;
+}
+
+// One site per thread: odd nx and sweep shape 0. Deviation storages are held to nine blocks per SM
+// without walls (56 registers), to seven with walls in index order (72).
+template <class L, typename S, bool WALLS, bool PART, bool FLAT>
+__global__ void __launch_bounds__(SWEEP_THREADS, WALLS ? (FLAT ? 7 : 1) : 9) k_sweep(const SweepArgs a)
 {
     using C = typename Store<S>::C;
     constexpr int Q = L::Q;
     const Geom& g = a.g;
-    const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned row = ((unsigned)z * (unsigned)g.ny + (unsigned)y) * (unsigned)g.nx;
-    const int xr = blockIdx.x * SWEEP_THREADS + threadIdx.x;
-    const bool valid = xr < g.nx;
-    const int x = valid ? xr : g.nx - 1;
-    const unsigned idx = row + (unsigned)x;
+    int x, y, z;
+    unsigned idx;
+    const bool valid = one_site<FLAT>(g, x, y, z, idx);
     const Nbr n = neighbours<WALLS>(g, x, y, z);
     // Owner tag and IS-source mask are loaded with the populations (no dependent round trip).
     unsigned tagx = TAG_FLUID, mask = 0;
@@ -1049,18 +1083,15 @@ __global__ void __launch_bounds__(PLAIN_THREADS) k_sweep_plain(const SweepArgs a
 // the phase's loads and stores on the one buffer (fin == fout). Deviation storages: at most
 // 56 registers (nine blocks per SM), measured 3 % faster than the unconstrained allocation at
 // the 512^3 suspension (FP32); FP64 keeps its registers.
-template <class L, typename S, bool WALLS, bool PART, int PHASE>
+template <class L, typename S, bool WALLS, bool PART, int PHASE, bool FLAT>
 __global__ void __launch_bounds__(SWEEP_THREADS, Store<S>::deviation ? 9 : 1) k_sweep_inplace(const SweepArgs a)
 {
     using C = typename Store<S>::C;
     constexpr int Q = L::Q;
     const Geom& g = a.g;
-    const int y = blockIdx.y, z = blockIdx.z;
-    const unsigned row = ((unsigned)z * (unsigned)g.ny + (unsigned)y) * (unsigned)g.nx;
-    const int xr = blockIdx.x * SWEEP_THREADS + threadIdx.x;
-    const bool valid = xr < g.nx;
-    const int x = valid ? xr : g.nx - 1;
-    const unsigned idx = row + (unsigned)x;
+    int x, y, z;
+    unsigned idx;
+    const bool valid = one_site<FLAT>(g, x, y, z, idx);
     const Nbr n = neighbours<WALLS>(g, x, y, z);
     unsigned tagx = TAG_FLUID, mask = 0;
     if constexpr (PART) {
@@ -1084,7 +1115,8 @@ __global__ void __launch_bounds__(SWEEP_THREADS, Store<S>::deviation ? 9 : 1) k_
 // One launch over a batch of cells: each block takes tiles of the schedule table (one, or a
 // stride of them in the persistent form) and runs the same per-site step as k_sweep with the
 // arguments of the tile's cell. Deviation storages without walls are held to nine blocks per SM
-// (56 registers, a few bytes of spills): the 64-cell ensemble's sweep 1.098 -> 1.065 ms.
+// (56 registers, a few bytes of spills): eight and ten blocks 0.971 and 1.112 ms against 0.958 ms at
+// the 64-cell ensemble.
 template <class L, typename S, bool WALLS, bool PART>
 __global__ void __launch_bounds__(SWEEP_THREADS, (Store<S>::deviation && !WALLS) ? 9 : 1)
     k_sweep_batch(const BatchSweepArgs b)
@@ -1107,12 +1139,27 @@ __global__ void __launch_bounds__(SWEEP_THREADS, (Store<S>::deviation && !WALLS)
         }
         const SweepArgs& a = sa;
         const Geom& g = a.g;
-        const int lw = t.z >> 16;
-        const int xr = t.y + (int)(threadIdx.x & ((1u << lw) - 1u));
-        const int yr = (t.z & 0xFFFF) + (int)(threadIdx.x >> lw);
-        const bool valid = xr < g.nx && yr < g.ny;
-        const int x = min(xr, g.nx - 1), y = min(yr, g.ny - 1), z = t.w;
-        const unsigned idx = ((unsigned)z * (unsigned)g.ny + (unsigned)y) * (unsigned)g.nx + (unsigned)x;
+        int x, y, z;
+        bool valid;
+        unsigned idx;
+        if (Store<S>::deviation && t.z < 0) {  // 128 sites in index order from t.y on
+            const unsigned at = (unsigned)t.y + threadIdx.x;
+            valid = at < g.N;
+            idx = min(at, g.N - 1u);
+            const unsigned row = idx / (unsigned)g.nx;
+            x = (int)(idx - row * (unsigned)g.nx);
+            z = (int)(row / (unsigned)g.ny);
+            y = (int)(row - (unsigned)z * (unsigned)g.ny);
+        } else {
+            const int lw = t.z >> 16;
+            const int xr = t.y + (int)(threadIdx.x & ((1u << lw) - 1u));
+            const int yr = (t.z & 0xFFFF) + (int)(threadIdx.x >> lw);
+            valid = xr < g.nx && yr < g.ny;
+            x = min(xr, g.nx - 1);
+            y = min(yr, g.ny - 1);
+            z = t.w;
+            idx = ((unsigned)z * (unsigned)g.ny + (unsigned)y) * (unsigned)g.nx + (unsigned)x;
+        }
         const Nbr n = neighbours<WALLS>(g, x, y, z);
         unsigned tagx = TAG_FLUID, mask = 0;
         if constexpr (PART) {
@@ -1604,16 +1651,27 @@ void launch_sweep_v(const SweepArgs& a, cudaStream_t s)
             return;
         }
     }
-    const dim3 grid((a.g.nx + SWEEP_THREADS - 1) / SWEEP_THREADS, a.g.ny, a.g.nz);
-    k_sweep<L, S, WALLS, PART><<<grid, SWEEP_THREADS, 0, s>>>(a);
+    if (index_order(a.g)) {
+        const unsigned blocks = (unsigned)(((size_t)a.g.N + SWEEP_THREADS - 1) / SWEEP_THREADS);
+        k_sweep<L, S, WALLS, PART, true><<<blocks, SWEEP_THREADS, 0, s>>>(a);
+    } else {
+        const dim3 grid((a.g.nx + SWEEP_THREADS - 1) / SWEEP_THREADS, a.g.ny, a.g.nz);
+        k_sweep<L, S, WALLS, PART, false><<<grid, SWEEP_THREADS, 0, s>>>(a);
+    }
 }
 
 template <class L, typename S, bool WALLS, bool PART>
 void launch_inplace_v(const SweepArgs& a, cudaStream_t s)
 {
-    const dim3 grid((a.g.nx + SWEEP_THREADS - 1) / SWEEP_THREADS, a.g.ny, a.g.nz);
-    if (a.aa == 1) k_sweep_inplace<L, S, WALLS, PART, 1><<<grid, SWEEP_THREADS, 0, s>>>(a);
-    else k_sweep_inplace<L, S, WALLS, PART, 2><<<grid, SWEEP_THREADS, 0, s>>>(a);
+    if (index_order(a.g)) {
+        const unsigned grid = (unsigned)(((size_t)a.g.N + SWEEP_THREADS - 1) / SWEEP_THREADS);
+        if (a.aa == 1) k_sweep_inplace<L, S, WALLS, PART, 1, true><<<grid, SWEEP_THREADS, 0, s>>>(a);
+        else k_sweep_inplace<L, S, WALLS, PART, 2, true><<<grid, SWEEP_THREADS, 0, s>>>(a);
+    } else {
+        const dim3 grid((a.g.nx + SWEEP_THREADS - 1) / SWEEP_THREADS, a.g.ny, a.g.nz);
+        if (a.aa == 1) k_sweep_inplace<L, S, WALLS, PART, 1, false><<<grid, SWEEP_THREADS, 0, s>>>(a);
+        else k_sweep_inplace<L, S, WALLS, PART, 2, false><<<grid, SWEEP_THREADS, 0, s>>>(a);
+    }
 }
 
 template <class L, typename S>

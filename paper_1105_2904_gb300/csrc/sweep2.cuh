@@ -32,7 +32,12 @@ template <> struct Pair<__half> {
     __device__ static float2 loadh(const __half* p) { return __half22float2(*reinterpret_cast<const __half2*>(p)); }
     __device__ static float loadh1(const __half* p) { return __half2float(*p); }
     __device__ static void storeh(__half* p, float2 h) { *reinterpret_cast<__half2*>(p) = __float22half2_rn(h); }
-    __device__ static float2 roundh(float2 h) { return __half22float2(__float22half2_rn(h)); }
+    __device__ static unsigned pack(float2 h)
+    {
+        const __half2 v = __float22half2_rn(h);
+        return *reinterpret_cast<const unsigned*>(&v);
+    }
+    __device__ static float2 unpack(unsigned u) { return __half22float2(*reinterpret_cast<const __half2*>(&u)); }
 };
 template <> struct Pair<__nv_bfloat16> {
     __device__ static float2 loadh(const __nv_bfloat16* p)
@@ -44,7 +49,12 @@ template <> struct Pair<__nv_bfloat16> {
     {
         *reinterpret_cast<__nv_bfloat162*>(p) = __float22bfloat162_rn(h);
     }
-    __device__ static float2 roundh(float2 h) { return __bfloat1622float2(__float22bfloat162_rn(h)); }
+    __device__ static unsigned pack(float2 h)
+    {
+        const __nv_bfloat162 v = __float22bfloat162_rn(h);
+        return *reinterpret_cast<const unsigned*>(&v);
+    }
+    __device__ static float2 unpack(unsigned u) { return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u)); }
 };
 
 // Component h (0: site x0, 1: site x0 + 1) of a pair.
@@ -242,6 +252,21 @@ __device__ __forceinline__ void kin2(const PKernF& k0, const PKernF& k1, float2 
     }
 }
 
+// Angular velocity and rigid velocity u_p + omega_p x r of both sites at their own places, each with
+// its own owner w0, w1.
+__device__ __forceinline__ void pair_kinematics(const Geom& g, int x0, int y, int z, unsigned w0, unsigned w1,
+                                                const PartView& pv, float2 om[3], float2 ux[3])
+{
+    if (!LBM_DCHECK(pv.status, w0 < (unsigned)pv.np)) w0 = 0u;
+    if (!LBM_DCHECK(pv.status, w1 < (unsigned)pv.np)) w1 = 0u;
+    const PKernF k0 = pv.pkf[w0];
+    const PKernF k1 = pv.pkf[w1];
+    float2 r[3], u[3];
+    lever_arm2(g, k0, k1, x0, y, z, r);
+    kin2(k0, k1, u, om);
+    rigid_velocity2(u, om, r, ux);
+}
+
 // c_i . v of a lattice direction on pairs (components 0 or +-1: adds only).
 template <class L, int i>
 __device__ __forceinline__ float2 cdot2(const float2 v[3])
@@ -264,9 +289,6 @@ __device__ __forceinline__ float2 cdot2(const float2 v[3])
     return r;
 }
 
-// The pending IS imposition (Eq. 12) for both sites of the pair, on packed pairs: the same
-// expression as substitute_is_dev (density carry: the pulled value is rho_I of its source),
-// each site with its own owner and IS-source mask. Warp-uniform; every lane calls it.
 // One site of the pair in the deviation units g of the scalar (one-site) code paths, and back:
 // HS pairs hold h = g / w (a value the scalar path leaves unchanged comes back within an FP32
 // rounding, far below the 16-bit storage's).
@@ -288,23 +310,22 @@ __device__ __forceinline__ void from_g_half(const float fs[], float2 f[])
     });
 }
 
-template <class L, bool WALLS, bool HS = false>
+// The pending IS imposition (Eq. 12) for both sites of the pair, on packed pairs: the same
+// expression as substitute_is_dev (density carry: the pulled value is rho_I of its source),
+// each site with its own owner and IS-source mask. Warp-uniform; every lane calls it. HS: om and
+// ux hold the angular and rigid velocities (pair_kinematics) wherever a mask is set; FP32 forms
+// them here.
+template <class L, bool WALLS, bool HS>
 __device__ __forceinline__ void substitute_is_dev2(const Geom& g, const Nbr& n0, const Nbr& n1, int x0, int y, int z,
-                                                   uint2 m, uint2 tags, const PartView& pv, float2 f[])
+                                                   uint2 m, uint2 tags, const PartView& pv, float2 om[3], float2 ux[3],
+                                                   float2 f[])
 {
     constexpr int Q = L::Q;
     const unsigned mm0 = m.x & ~MASK_OTHER, mm1 = m.y & ~MASK_OTHER;
     const unsigned wm = __reduce_or_sync(__activemask(), mm0 | mm1);
     if (wm) {
-        unsigned w0 = mm0 ? (tags.x & PID_MASK) : 0u, w1 = mm1 ? (tags.y & PID_MASK) : 0u;
-        if (!LBM_DCHECK(pv.status, w0 < (unsigned)pv.np)) w0 = 0u;
-        if (!LBM_DCHECK(pv.status, w1 < (unsigned)pv.np)) w1 = 0u;
-        const PKernF k0 = pv.pkf[w0];
-        const PKernF k1 = pv.pkf[w1];
-        float2 r[3], u[3], om[3], ux[3];
-        lever_arm2(g, k0, k1, x0, y, z, r);
-        kin2(k0, k1, u, om);
-        rigid_velocity2(u, om, r, ux);
+        if constexpr (!HS)
+            pair_kinematics(g, x0, y, z, mm0 ? (tags.x & PID_MASK) : 0u, mm1 ? (tags.y & PID_MASK) : 0u, pv, om, ux);
         float2 b[3];  // u(x) + u(x) x omega
         b[0] = add2(ux[0], sub2(mul2(ux[1], om[2]), mul2(ux[2], om[1])));
         b[1] = add2(ux[1], sub2(mul2(ux[2], om[0]), mul2(ux[0], om[2])));
@@ -397,22 +418,18 @@ __device__ __forceinline__ void eq_face_half(const float u[3], float drho, float
 
 // BS transfer (Eqs. 5-7) of the BS sites of the pair on packed pairs: the same expression
 // as bs_transfer_dev; each BS site takes f^eq(rho_B, u_p + omega_p x r) and writes its
-// per-site record.
-template <class L, bool BRICK, bool HS = false>
+// per-site record. HS: ub holds the rigid velocities.
+template <class L, bool BRICK, bool HS>
 __device__ __forceinline__ void bs_transfer_dev2(const SweepArgs& a, int x0, int y, int z, unsigned idx, uint2 tags,
-                                                 bool bs0, bool bs1, float2 mrho, float2 mj0, float2 mj1, float2 mj2,
-                                                 float2 f[])
+                                                 bool bs0, bool bs1, float2 ub[3], float2 mrho, float2 mj0, float2 mj1,
+                                                 float2 mj2, float2 f[])
 {
     constexpr int Q = L::Q;
-    unsigned p0 = tags.x & PID_MASK, p1 = tags.y & PID_MASK;
-    if (!LBM_DCHECK(a.pv.status, !bs0 || p0 < (unsigned)a.pv.np)) p0 = 0u;
-    if (!LBM_DCHECK(a.pv.status, !bs1 || p1 < (unsigned)a.pv.np)) p1 = 0u;
-    const PKernF k0 = a.pv.pkf[bs0 ? p0 : p1];
-    const PKernF k1 = a.pv.pkf[bs1 ? p1 : p0];
-    float2 r[3], u[3], om[3], ub[3];
-    lever_arm2(a.g, k0, k1, x0, y, z, r);
-    kin2(k0, k1, u, om);
-    rigid_velocity2(u, om, r, ub);
+    if constexpr (!HS) {
+        const unsigned p0 = tags.x & PID_MASK, p1 = tags.y & PID_MASK;
+        float2 om[3];
+        pair_kinematics(a.g, x0, y, z, bs0 ? p0 : p1, bs1 ? p1 : p0, a.pv, om, ub);
+    }
     const float2 rho = add2(mrho, p2(1.0f));
     const float2 usq15 = mul2(p2(1.5f), fma2(ub[2], ub[2], fma2(ub[1], ub[1], mul2(ub[0], ub[0]))));
     {   // (HS: in h units, without the w_i factor)
@@ -450,17 +467,25 @@ __device__ __forceinline__ void bs_transfer_dev2(const SweepArgs& a, int x0, int
     if (bs1) sc[1] = make_float4(dv[0].y, dv[1].y, dv[2].y, __uint_as_float(tags.y));
 }
 
-// One block: BX threads along x (2 BX sites) times 128 / BX rows of one z-plane, five blocks per
-// SM (96 registers, no spills). The 16-bit storages compute in their stored units
-// h = (f - w) / w, which saves the scaling of every load and store (FP16 sweep 3.350 -> 3.324 ms
-// at the 512^3 suspension); with that and the IS-source masks loaded only at solid pairs they
-// run best at five blocks as well (3.225 ms at six blocks and 80 registers, with spills; seven
-// blocks spill far more), as FP32 always did (six blocks measured slower).
+// FP32 storage: rows of the populations brought into L2 ahead of the blocks in flight, some
+// PREFETCH_SITES sites (one bulk prefetch per direction and group of rows, by the group's first
+// block), shorten the wait for DRAM and are read in long bursts: 256^3 suspension 0.438 -> 0.424
+// ms, 512^3 3.52 -> 3.50 ms. Further ahead they are evicted before use (two and five times the
+// distance: 0.509 and 0.584 ms). The 16-bit sweep gains nothing (3.16 -> 3.20 ms), and boxes that
+// stay in L2 from step to step have no use for it.
+constexpr unsigned PREFETCH_SITES = 131072, PREFETCH_MIN_SITES = 1u << 20;
+
+// One block: BX threads along x (2 BX sites) times 64 / BX rows of one z-plane (one row for BX = 128),
+// twenty warps per SM (96 registers; twenty-four with spills were slower). Blocks of two warps
+// instead of four leave fewer slots waiting for a block's last warp: 512^3 FP32 3.523 -> 3.491 ms,
+// FP16 3.158 -> 3.134 ms (one warp: 3.503, 3.154 ms). The 16-bit storages compute in their
+// stored units h = (f - w) / w, which saves the scaling of every load and store.
+__host__ __device__ constexpr int pair_threads(int bx) { return bx > 64 ? bx : 64; }
 template <class L, typename S, bool WALLS, bool PART, int BX>
-__global__ void __launch_bounds__(SWEEP_THREADS, 5) k_sweep2(const SweepArgs a)
+__global__ void __launch_bounds__(pair_threads(BX), 640 / pair_threads(BX)) k_sweep2(const SweepArgs a)
 {
     constexpr int Q = L::Q;
-    constexpr int BY = SWEEP_THREADS / BX;
+    constexpr int BY = pair_threads(BX) / BX;
     const Geom& g = a.g;
     const int tx = (int)threadIdx.x % BX, ty = (int)threadIdx.x / BX;
     const int xr = (int)blockIdx.x * (2 * BX) + 2 * tx;
@@ -469,6 +494,20 @@ __global__ void __launch_bounds__(SWEEP_THREADS, 5) k_sweep2(const SweepArgs a)
     const bool valid = xr < g.nx && yr < g.ny;
     const int x0 = min(xr, g.nx - 2), y = min(yr, g.ny - 1);
     const unsigned idx = ((unsigned)z * (unsigned)g.ny + (unsigned)y) * (unsigned)g.nx + (unsigned)x0;
+    if (sizeof(S) == 4 && blockIdx.x == 0 && a.ahead && threadIdx.x < Q) {
+        unsigned gy = blockIdx.y + (unsigned)a.ahead;
+        const unsigned zz = blockIdx.z + gy / gridDim.y;
+        gy %= gridDim.y;
+        if (zz < gridDim.z) {
+            const size_t first = ((size_t)(zz * (unsigned)g.ny + gy * BY)) * (unsigned)g.nx;
+            const unsigned n = min((unsigned)BY, (unsigned)g.ny - gy * BY) * (unsigned)g.nx;
+            const S* q = (const S*)a.fin + (size_t)threadIdx.x * g.N + first;
+            // from the first 16-byte boundary inside the rows to the last
+            const size_t lo = ((size_t)q + 15) & ~(size_t)15, hi = (size_t)(q + n) & ~(size_t)15;
+            if (lo < hi)
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo), "r"((unsigned)(hi - lo)) : "memory");
+        }
+    }
     Nbr n0, n1;
     pair_neighbours<WALLS>(g, x0, y, z, n0, n1);
     // 16-bit storages: the pair values stay in the stored units h = (f - w) / w throughout
@@ -486,10 +525,27 @@ __global__ void __launch_bounds__(SWEEP_THREADS, 5) k_sweep2(const SweepArgs a)
     // memory rather than issue, measured 3.573 -> 3.784 ms, so FP32 loads them with the tags)
     if constexpr (PART && HS)
         if (tg.x != TAG_FLUID || tg.y != TAG_FLUID) mk = *reinterpret_cast<const uint2*>(a.pv.ismask + idx);
-    if constexpr (PART) {
+    // The 16-bit sweep, bound by instructions and their latency, loads a pair's particle records and
+    // forms its rigid velocity once for the imposition and the BS transfer (512^3 suspension, FP16:
+    // 3.14 -> 2.91 ms). FP32, bound by memory, is slower that way (3.49 -> 3.71 ms): its warps then
+    // wait for the records wherever they cross a particle, also where no mask is set.
+    float2 ux[3];
+    if constexpr (PART && HS) {
+        const bool s0 = tg.x != TAG_FLUID, s1 = tg.y != TAG_FLUID;
+        if (__any_sync(0xffffffffu, s0 || s1)) {
+            // (a fluid site of a solid pair takes its neighbour's owner, a fluid pair particle 0)
+            const unsigned w0 = s0 ? tg.x & PID_MASK : (s1 ? tg.y & PID_MASK : 0u);
+            float2 om[3];
+            pair_kinematics(g, x0, y, z, w0, s1 ? tg.y & PID_MASK : w0, a.pv, om, ux);
+            if (*a.pv.pending)
+                substitute_is_dev2<L, WALLS, HS>(g, n0, n1, x0, y, z, make_uint2(s0 ? mk.x : 0u, s1 ? mk.y : 0u), tg, a.pv, om,
+                                                 ux, f);
+        }
+    } else if constexpr (PART) {
         if (*a.pv.pending) {
             const uint2 m = make_uint2(tg.x != TAG_FLUID ? mk.x : 0u, tg.y != TAG_FLUID ? mk.y : 0u);
-            substitute_is_dev2<L, WALLS, HS>(g, n0, n1, x0, y, z, m, tg, a.pv, f);
+            float2 om[3], u[3];
+            substitute_is_dev2<L, WALLS, HS>(g, n0, n1, x0, y, z, m, tg, a.pv, om, u, f);
         }
     }
     // A moving wall acts on the bounced value after the IS imposition it may have received.
@@ -506,7 +562,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS, 5) k_sweep2(const SweepArgs a)
     if constexpr (PART) {
         const bool bs0 = valid && (tg.x >> 30) == CLS_BS, bs1 = valid && (tg.y >> 30) == CLS_BS;
         if (bs0 || bs1)
-            bs_transfer_dev2<L, std::is_same<S, float>::value, HS>(a, x0, y, z, idx, tg, bs0, bs1, mrho, mj0, mj1,
+            bs_transfer_dev2<L, std::is_same<S, float>::value, HS>(a, x0, y, z, idx, tg, bs0, bs1, ux, mrho, mj0, mj1,
                                                                   mj2, f);
         is0 = (tg.x >> 30) == CLS_IS;
         is1 = (tg.y >> 30) == CLS_IS;
@@ -527,25 +583,33 @@ __global__ void __launch_bounds__(SWEEP_THREADS, 5) k_sweep2(const SweepArgs a)
         // density carry: an IS site stores its post-collision density (the sum of its values
         // as stored) in every slot
         float2 dens = p2(0.0f);
-        sfor<0, Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            if constexpr (HS) dens = fma2(p2((float)L::w(i)), Pair<S>::roundh(f[i]), dens);
-            else dens = add2(dens, Pair<S>::round(f[i], (float)L::w(i)));
-        });
-        sfor<0, Q>([&](auto ic) {
-            constexpr int i = decltype(ic)::value;
-            float2 v = f[i];
-            if constexpr (HS) {
-                const float2 dh = mul2(dens, p2(1.0f / (float)L::w(i)));
-                if (is0) v.x = dh.x;
-                if (is1) v.y = dh.y;
-                Pair<S>::storeh(fout + (size_t)i * N + idx, v);
-            } else {
+        if constexpr (HS) {
+            // on the packed values, by a lane mask (2.968 -> 2.931 ms against selects of both halves)
+            unsigned s[Q];
+            sfor<0, Q>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                s[i] = Pair<S>::pack(f[i]);
+                dens = fma2(p2((float)L::w(i)), Pair<S>::unpack(s[i]), dens);
+            });
+            const unsigned take = (is0 ? 0xFFFFu : 0u) | (is1 ? 0xFFFF0000u : 0u);
+            sfor<0, Q>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                const unsigned d = Pair<S>::pack(mul2(dens, p2(1.0f / (float)L::w(i))));
+                *reinterpret_cast<unsigned*>(fout + (size_t)i * N + idx) = (s[i] & ~take) | (d & take);
+            });
+        } else {
+            sfor<0, Q>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                dens = add2(dens, Pair<S>::round(f[i], (float)L::w(i)));
+            });
+            sfor<0, Q>([&](auto ic) {
+                constexpr int i = decltype(ic)::value;
+                float2 v = f[i];
                 if (is0) v.x = dens.x;
                 if (is1) v.y = dens.y;
                 Pair<S>::store(fout + (size_t)i * N + idx, v, (float)L::w(i));
-            }
-        });
+            });
+        }
     } else {
         sfor<0, Q>([&](auto ic) {
             constexpr int i = decltype(ic)::value;
@@ -556,15 +620,16 @@ __global__ void __launch_bounds__(SWEEP_THREADS, 5) k_sweep2(const SweepArgs a)
 }
 
 template <class L, typename S, bool WALLS, bool PART>
-void launch_sweep2_v(const SweepArgs& a, int bx, cudaStream_t s)
+void launch_sweep2_v(SweepArgs a, int bx, cudaStream_t s)
 {
-    const int by = SWEEP_THREADS / bx;
+    const int threads = pair_threads(bx), by = threads / bx;
+    a.ahead = a.g.N >= PREFETCH_MIN_SITES ? (int)(PREFETCH_SITES / ((unsigned)a.g.nx * (unsigned)by)) + 1 : 0;
     const dim3 grid((a.g.nx + 2 * bx - 1) / (2 * bx), (a.g.ny + by - 1) / by, a.g.nz);
     switch (bx) {
-    case 16: k_sweep2<L, S, WALLS, PART, 16><<<grid, SWEEP_THREADS, 0, s>>>(a); break;
-    case 32: k_sweep2<L, S, WALLS, PART, 32><<<grid, SWEEP_THREADS, 0, s>>>(a); break;
-    case 64: k_sweep2<L, S, WALLS, PART, 64><<<grid, SWEEP_THREADS, 0, s>>>(a); break;
-    default: k_sweep2<L, S, WALLS, PART, 128><<<grid, SWEEP_THREADS, 0, s>>>(a); break;
+    case 16: k_sweep2<L, S, WALLS, PART, 16><<<grid, threads, 0, s>>>(a); break;
+    case 32: k_sweep2<L, S, WALLS, PART, 32><<<grid, threads, 0, s>>>(a); break;
+    case 64: k_sweep2<L, S, WALLS, PART, 64><<<grid, threads, 0, s>>>(a); break;
+    default: k_sweep2<L, S, WALLS, PART, 128><<<grid, threads, 0, s>>>(a); break;
     }
 }
 
