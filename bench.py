@@ -445,7 +445,8 @@ def run_ours(args):
                 "traffic": (rec["dram_bytes_per_site"] * N if rec else None),
                 "kernel": ("k_sweep_inplace (neighbour and local phases in turn, one buffer): fused in-place "
                            "stream" if inplace else
-                           ("k_sweep2 (two sites per thread, %d threads along x)" % shape if two_site else "k_sweep")
+                           ("k_sweep2 (two sites per thread, %d threads along x)" % shape if two_site else
+                            "k_impose_plain, k_sweep_plain, k_solid_plain" if args.precision == "fp64" else "k_sweep")
                            + ": fused pull-stream")
                           + " + IS imposition + collide + BS transfer",
                 "algorithmic_bytes_per_launch": algo_bytes, "sweep_ms": prof["sweep_ms"],

@@ -216,8 +216,8 @@ lbm_status lbm_profile_steps(lbm_ctx* ctx, int n, double out_ms[3]);
  * describes a serial algorithm; results agree to FP32 rounding). For the
  * FP32 / FP16 / BF16 storages on a lattice with even nx, threads_x = 16, 32, 64 or 128
  * selects the two-site kernel (each thread updates the sites x, x + 1 with paired 8- or
- * 4-byte accesses and packed FP32 pair arithmetic; blocks of 128 threads, threads_x of them
- * along x, 128 / threads_x rows); 0 selects the one-site kernel; -1 (the default) picks
+ * 4-byte accesses and packed FP32 pair arithmetic; blocks of 64 threads, 128 for threads_x =
+ * 128, threads_x of them along x); 0 selects the one-site kernel; -1 (the default) picks
  * the two-site kernel with 16 threads along x (the one-site kernel where nx is odd). FP64
  * storage always uses the one-site kernel. Drops the captured step graphs. LBM_E_INVALID for
  * other values. */
@@ -340,8 +340,9 @@ lbm_status lbm_bs_exchange_noalloc(int lattice, int nx, int ny, int nz, const in
  * its own tau, body force and particles) advanced together. The paper simulates one box at
  * a time; the batch only changes how the work is launched: every step runs one sweep
  * launch over all cells (a schedule table of 128-thread tiles, each tile one rectangle of
- * one x-y plane of one cell) and one launch per particle-phase kernel (the cell as the
- * second grid index), captured in CUDA graphs of one or several steps. Each cell's result
+ * one x-y plane of one cell; cells whose tiles would leave over a tenth of their threads idle
+ * are swept in index order, 128 consecutive sites a tile) and one launch per particle-phase
+ * kernel (the cell as the second grid index; FP64 storage three for the sweep), captured in CUDA graphs of one or several steps. Each cell's result
  * is bit for bit the result of stepping it alone with the one-site sweep kernel
  * (lbm_set_sweep_shape(ctx, 0)); the batch sweep is that kernel. */
 
