@@ -277,8 +277,8 @@ constexpr long long FUSED_WEIGHTS = 262144;
 constexpr size_t FUSED_SMEM = 160 * 1024;
 
 __host__ __device__ constexpr int pad16(int n) { return (n + 15) / 16 * 16; }
-// Row stride of a bfloat16 tile in shared memory: 8 n + 4 words with n odd or even, so the eight
-// rows of a fragment fall into different banks.
+// Row stride of a bfloat16 tile in shared memory, an odd multiple of four words: the eight rows of a
+// fragment fall into different banks.
 __host__ __device__ constexpr int tile_ld(int n) { return pad16(n) + 8; }
 __host__ __device__ constexpr long long frag_elems(int k, int n) { return (long long)((n + 7) / 8) * ((k + 15) / 16) * 128; }
 // Position of B(k, n) among the fragments of a K x N operand (m16n8k16, "col" B).
