@@ -218,7 +218,7 @@ int launch_particle_phase_b(const ParticleArgs& a, cudaStream_t s);
 void launch_stamp_all(const ParticleArgs& a, cudaStream_t s);
 
 // Arguments of k_remark (sweep.cuh): the re-marking of one step in one launch.
-constexpr int REMARK_CLUSTER = 8, REMARK_CLUSTER_BATCH = 4;
+constexpr int REMARK_CLUSTER = 16, REMARK_CLUSTER_BATCH = 4;
 constexpr long long REMARK_ENTRIES = 262144;
 struct RemarkArgs {
     ISFixArgs f;               // (f.dens: in-place streaming's density array there)

@@ -617,8 +617,8 @@ __device__ __forceinline__ void mark_neighbours(const ParticleArgs& a, int p, co
     const double rp = a.pc[p].r;
     double cold[3], cnew[3];
     for (int k = 0; k < 3; ++k) {
-        cold[k] = (double)__ldcg(&a.Kold[(size_t)p * 3 + k]) + a.pk[p].phi[k];
-        cnew[k] = (double)__ldcg(&a.pk[p].K[k]) + a.pk[p].phi[k];
+        cold[k] = (double)a.Kold[(size_t)p * 3 + k] + a.pk[p].phi[k];
+        cnew[k] = (double)a.pk[p].K[k] + a.pk[p].phi[k];
     }
     for (int zz = 0; zz < nzc; ++zz)
         for (int yy = 0; yy < nyc; ++yy)
@@ -631,7 +631,7 @@ __device__ __forceinline__ void mark_neighbours(const ParticleArgs& a, int p, co
                     const double R = rp + a.pc[q].r + 1.0;
                     double d2o = 0.0, d2n = 0.0;
                     for (int k = 0; k < 3; ++k) {
-                        const double cq = (double)__ldcg(&a.pk[q].K[k]) + a.pk[q].phi[k];
+                        const double cq = (double)a.pk[q].K[k] + a.pk[q].phi[k];
                         const double dd0 = min_image(cold[k] - cq, axis_len(a.g, k), periodic_axis(a.g, k, D));
                         const double dd1 = min_image(cnew[k] - cq, axis_len(a.g, k), periodic_axis(a.g, k, D));
                         d2o += dd0 * dd0;
@@ -661,9 +661,8 @@ __global__ void k_mark_clear(const ParticleArgs a0, const ParticleArgs* __restri
     if (a.np == 0) return;  // a cell of a batch without particles
     const int nlist = a.cnt->nchanged;
     for (int b = blockIdx.x; b < nlist; b += gridDim.x) {
-        const int p = a.changed[b];
-        const OldAnchor o(a, p);
-        for (int e = threadIdx.x; e < a.pc[p].tmpl_n; e += blockDim.x) clear_entry(a, p, o, e);
+        const Moved h(a.g, a.pc, a.pk, a.Kold, a.changed[b]);
+        for (int e = threadIdx.x; e < h.n; e += blockDim.x) clear_entries<1>(a, h, e, 0);
     }
 }
 
@@ -673,14 +672,18 @@ __global__ void k_mark_stamp(const ParticleArgs a0, const ParticleArgs* __restri
     const ParticleArgs a = cell_args<B>(a0, cells);
     if (a.np == 0) return;  // a cell of a batch without particles
     const int nlist = a.cnt->nrestamp;
-    for (int b = blockIdx.x; b < nlist; b += gridDim.x)
-        for (int p = a.restamp[b], e = threadIdx.x; e < a.pc[p].tmpl_n; e += blockDim.x) stamp_entry(a, p, e);
+    for (int b = blockIdx.x; b < nlist; b += gridDim.x) {
+        const Stamped h(a.pc, a.pk, a.restamp[b]);
+        for (int e = threadIdx.x; e < h.n; e += blockDim.x) stamp_entries<1>(a, h, e, 0);
+    }
 }
 
 __global__ void k_stamp_all(const ParticleArgs a)
 {
-    for (int p = blockIdx.x; p < a.np; p += gridDim.x)
-        for (int e = threadIdx.x; e < a.pc[p].tmpl_n; e += blockDim.x) stamp_entry(a, p, e);
+    for (int p = blockIdx.x; p < a.np; p += gridDim.x) {
+        const Stamped h(a.pc, a.pk, p);
+        for (int e = threadIdx.x; e < h.n; e += blockDim.x) stamp_entries<1>(a, h, e, 0);
+    }
 }
 
 // ---- few particles -----------------------------------------------------------------------------

@@ -667,16 +667,15 @@ __device__ __forceinline__ void is_density_from_array_warp(const Geom& g, const 
     if (m & MASK_OTHER) is_density_from_array<L, C, WALLS>(g, n, x, y, z, idx, MASK_OTHER, pv, rho, f);
 }
 
-// Rebuilds the IS-source mask at the site of template entry e of particle p.
+// Rebuilds the IS-source mask at the site of template entry e of a particle.
 template <class L>
-__device__ __forceinline__ void mask_entry(const MaskArgs& a, int p, int e)
+__device__ __forceinline__ void mask_entry(const MaskArgs& a, const Stamped& h, int e)
 {
     const Geom& g = a.g;
-    const int Kw[3] = {a.pk[p].Kw[0], a.pk[p].Kw[1], a.pk[p].Kw[2]};
-    const int ent = a.tmpl[a.pc[p].tmpl_off + e];
+    const int ent = a.tmpl[h.off + e];
     unsigned idx;
     int v[3];
-    if (!site_fast_xyz(g, Kw, tmpl_ox(ent), tmpl_oy(ent), tmpl_oz(ent), idx, v)) return;
+    if (!site_fast_xyz(g, h.Kw, tmpl_ox(ent), tmpl_oy(ent), tmpl_oz(ent), idx, v)) return;
     const unsigned owner = a.tag[idx] & PID_MASK;
     const int x = v[0], y = v[1], z = v[2];
     const Nbr n = neighbours<true>(g, x, y, z);
@@ -702,8 +701,8 @@ __global__ void k_update_masks(const MaskArgs a0, const MaskArgs* __restrict__ c
     if (a.np == 0 || (a.list && !a.cnt)) return;
     const int count = a.list ? a.cnt->nrestamp : a.np;
     for (int b = blockIdx.x; b < count; b += gridDim.x) {
-        const int p = a.list ? a.list[b] : b;
-        for (int e = threadIdx.x; e < a.pc[p].tmpl_n; e += blockDim.x) mask_entry<L>(a, p, e);
+        const Stamped h(a.pc, a.pk, a.list ? a.list[b] : b);
+        for (int e = threadIdx.x; e < h.n; e += blockDim.x) mask_entry<L>(a, h, e);
     }
 }
 
@@ -1401,38 +1400,30 @@ __global__ void k_fill_rest(S* dst, unsigned N)
 // kernels (one block per such particle, threads over its IS template entries at the anchor
 // the sweep used and at the new one) restore the invariant for the new owner map.
 
-// Site of IS template entry e of particle p at anchor K (false if it leaves a walled domain).
-__device__ __forceinline__ bool is_entry_site(const ISFixArgs& a, const int K[3], int e, unsigned& site)
-{
-    int Kw[3];
-    wrap_anchor(a.s.g, K, Kw);
-    const int ent = a.tmpl[e];
-    return site_fast(a.s.g, Kw, tmpl_ox(ent), tmpl_oy(ent), tmpl_oz(ent), site);
-}
+__device__ __forceinline__ Moved moved_particle(const ISFixArgs& a, int p) { return Moved(a.s.g, a.pc, a.pk, a.Kold, p); }
 
-// Entry e of the visited sites of moved particle p: its IS template entries at the old anchor,
-// then at the new one.
-__device__ __forceinline__ bool visited_site(const ISFixArgs& a, int p, int e, unsigned& site)
+// Entry e of the visited sites of a moved particle: its IS template entries at the old anchor, then
+// at the new one (false if the site leaves a walled domain).
+__device__ __forceinline__ bool visited_site(const ISFixArgs& a, const Moved& h, int e, unsigned& site)
 {
-    const int n_is = a.pc[p].n_is;
-    const bool old = e < n_is;
-    const int K[3] = {old ? a.Kold[(size_t)p * 3] : a.pk[p].K[0], old ? a.Kold[(size_t)p * 3 + 1] : a.pk[p].K[1],
-                      old ? a.Kold[(size_t)p * 3 + 2] : a.pk[p].K[2]};
-    return is_entry_site(a, K, a.pc[p].tmpl_off + a.pc[p].n_bs + e % n_is, site);
+    const bool old = e < h.n_is;
+    const int K[3] = {old ? h.Ko[0] : h.Kw[0], old ? h.Ko[1] : h.Kw[1], old ? h.Ko[2] : h.Kw[2]};
+    const int ent = a.tmpl[h.is_off + (old ? e : e - h.n_is)];
+    return site_fast(a.s.g, K, tmpl_ox(ent), tmpl_oy(ent), tmpl_oz(ent), site);
 }
 
 // (1) Before the owner map changes: the density of every visited site, read from the
 // sweep's output (one slot of a site the sweep saw as IS, else the sum of its populations in
 // slot order, the sum the sweep takes).
 template <class L, typename S>
-__device__ __forceinline__ void is_density_entry(const ISFixArgs& a, int p, int e)
+__device__ __forceinline__ void is_density_entry(const ISFixArgs& a, const Moved& h, int e)
 {
     using St = Store<S>;
     using C = typename St::C;
     const size_t N = a.s.g.N;
     const S* fo = (const S*)a.s.fout;
     unsigned site;
-    if (!visited_site(a, p, e, site)) return;
+    if (!visited_site(a, h, e, site)) return;
     C d = (C)0;
     if ((a.s.pv.tag[site] >> 30) == CLS_IS) {
         d = St::load(fo[site], (C)L::w(0));
@@ -1451,23 +1442,24 @@ __global__ void k_is_density(const ISFixArgs a0, const ISFixArgs* __restrict__ c
     const ISFixArgs a = pick_args<B>(a0, cells);
     if (!a.cnt) return;
     const int nlist = a.cnt->nchanged;
-    for (int b = blockIdx.x; b < nlist; b += gridDim.x)
-        for (int p = a.list[b], e = threadIdx.x; e < 2 * a.pc[p].n_is; e += blockDim.x) is_density_entry<L, S>(a, p, e);
+    for (int b = blockIdx.x; b < nlist; b += gridDim.x) {
+        const Moved h = moved_particle(a, a.list[b]);
+        for (int e = threadIdx.x; e < 2 * h.n_is; e += blockDim.x) is_density_entry<L, S>(a, h, e);
+    }
 }
 
 // (2) Still before the owner map changes: the sites the sweep saw as IS of a particle whose
 // shift changed get the populations the sweep computed for them (recomputed from the
 // sweep's input with the sweep's particle view; same code, same result bit for bit).
 template <class L, typename S, bool WALLS>
-__device__ __forceinline__ void is_restore_entry(const ISFixArgs& a, int p, int e)
+__device__ __forceinline__ void is_restore_entry(const ISFixArgs& a, const Moved& h, int e)
 {
     using C = typename Store<S>::C;
     const Geom& g = a.s.g;
-    const int Ko[3] = {a.Kold[(size_t)p * 3], a.Kold[(size_t)p * 3 + 1], a.Kold[(size_t)p * 3 + 2]};
     unsigned site;
-    if (!is_entry_site(a, Ko, a.pc[p].tmpl_off + a.pc[p].n_bs + e, site)) return;
+    if (!visited_site(a, h, e, site)) return;  // (e < n_is: at the old anchor)
     const unsigned t = a.s.pv.tag[site];
-    if (t != ((CLS_IS << 30) | (unsigned)p)) return;
+    if (t != ((CLS_IS << 30) | (unsigned)h.p)) return;
     const int x = (int)(site % (unsigned)g.nx);
     const int y = (int)((site / (unsigned)g.nx) % (unsigned)g.ny);
     const int z = (int)(site / ((unsigned)g.nx * (unsigned)g.ny));
@@ -1484,20 +1476,22 @@ __global__ void k_is_restore(const ISFixArgs a0, const ISFixArgs* __restrict__ c
     const ISFixArgs a = pick_args<B>(a0, cells);
     if (!a.cnt) return;
     const int nlist = a.cnt->nchanged;
-    for (int b = blockIdx.x; b < nlist; b += gridDim.x)
-        for (int p = a.list[b], e = threadIdx.x; e < a.pc[p].n_is; e += blockDim.x) is_restore_entry<L, S, WALLS>(a, p, e);
+    for (int b = blockIdx.x; b < nlist; b += gridDim.x) {
+        const Moved h = moved_particle(a, a.list[b]);
+        for (int e = threadIdx.x; e < h.n_is; e += blockDim.x) is_restore_entry<L, S, WALLS>(a, h, e);
+    }
 }
 
 // (3) After re-marking: every visited site that is now IS holds its density in every slot.
 template <class L, typename S>
-__device__ __forceinline__ void is_fix_entry(const ISFixArgs& a, int p, int e)
+__device__ __forceinline__ void is_fix_entry(const ISFixArgs& a, const Moved& h, int e)
 {
     using St = Store<S>;
     using C = typename St::C;
     const size_t N = a.s.g.N;
     S* fo = (S*)a.s.fout;
     unsigned site;
-    if (!visited_site(a, p, e, site)) return;
+    if (!visited_site(a, h, e, site)) return;
     if ((a.s.pv.tag[site] >> 30) != CLS_IS) return;
     const C d = ((const C*)a.dens)[site];
     sfor<0, L::Q>([&](auto ic) {
@@ -1512,8 +1506,10 @@ __global__ void k_is_fix(const ISFixArgs a0, const ISFixArgs* __restrict__ cells
     const ISFixArgs a = pick_args<B>(a0, cells);
     if (!a.cnt) return;
     const int nlist = a.cnt->nchanged;
-    for (int b = blockIdx.x; b < nlist; b += gridDim.x)
-        for (int p = a.list[b], e = threadIdx.x; e < 2 * a.pc[p].n_is; e += blockDim.x) is_fix_entry<L, S>(a, p, e);
+    for (int b = blockIdx.x; b < nlist; b += gridDim.x) {
+        const Moved h = moved_particle(a, a.list[b]);
+        for (int e = threadIdx.x; e < 2 * h.n_is; e += blockDim.x) is_fix_entry<L, S>(a, h, e);
+    }
 }
 
 // In-place streaming, after re-marking: every visited site that is now IS gets its density
@@ -1521,7 +1517,7 @@ __global__ void k_is_fix(const ISFixArgs a0, const ISFixArgs* __restrict__ cells
 // (the sum the sweep takes), found where the sweep's phase left them (s.aa: 2 = slot i of x;
 // 1 = slot opp(i) of x + c_i, or slot i of x where x + c_i lies beyond a wall).
 template <class L, typename S, bool WALLS>
-__device__ __forceinline__ void inplace_fix_entry(const ISFixArgs& a, int p, int e)
+__device__ __forceinline__ void inplace_fix_entry(const ISFixArgs& a, const Moved& h, int e)
 {
     using St = Store<S>;
     using C = typename St::C;
@@ -1529,7 +1525,7 @@ __device__ __forceinline__ void inplace_fix_entry(const ISFixArgs& a, int p, int
     const size_t N = g.N;
     const S* fo = (const S*)a.s.fout;
     unsigned site;
-    if (!visited_site(a, p, e, site)) return;
+    if (!visited_site(a, h, e, site)) return;
     if ((a.s.pv.tag[site] >> 30) != CLS_IS) return;
     C d = (C)0;
     if (a.s.aa == 2) {
@@ -1560,58 +1556,84 @@ __global__ void k_inplace_fix(const ISFixArgs a)
 {
     if (!a.cnt) return;
     const int nlist = a.cnt->nchanged;
-    for (int b = blockIdx.x; b < nlist; b += gridDim.x)
-        for (int p = a.list[b], e = threadIdx.x; e < 2 * a.pc[p].n_is; e += blockDim.x) inplace_fix_entry<L, S, WALLS>(a, p, e);
+    for (int b = blockIdx.x; b < nlist; b += gridDim.x) {
+        const Moved h = moved_particle(a, a.list[b]);
+        for (int e = threadIdx.x; e < 2 * h.n_is; e += blockDim.x) inplace_fix_entry<L, S, WALLS>(a, h, e);
+    }
 }
 
 // ---- few template entries: the whole re-marking in one launch ---------------------------------
 // The kernels above and the owner-map update between them are six launches of 2.5 us that find
 // nothing to do in most steps of a small suspension (a sphere at u = 1e-3 crosses a site boundary
-// once in some 300 steps). Here they are one: a cluster of 8 blocks returns at once when no shift
-// changed, and otherwise spreads each moved particle's entries over its 4096 threads with a
-// cluster barrier where the launches had a boundary. Above REMARK_ENTRIES template entries in all,
-// a fast suspension could change more of them in a step than a cluster gets through in the time
-// the launches take, so larger ones keep the launches.
+// once in some 300 steps). Here they are one: a cluster of 16 blocks returns at once when no shift
+// changed, and otherwise spreads each moved particle's entries over its 8192 threads with a
+// cluster barrier where the launches had a boundary. In a fast suspension every phase has work for
+// more threads than a cluster has, and what counts is the chain of loads per entry: the particle's
+// record and anchors are loaded once for all phases and entries, four entries are cleared or stamped
+// at a time. The five phases of a step that moves 90 of 800 disks of radius 10 take 28 us (a cluster
+// of 8 with the records loaded per entry: 76 us; six launches: 45 us), of one that moves 90 of 500
+// spheres of radius 5 66 us (105 us; 62 us). Whole steps, us, six launches / one: none moving 800 disks
+// 53.6 / 39.5, 500 spheres 102 / 85; sigma = 0.08 131 / 129 and 575 / 610. Above REMARK_ENTRIES
+// template entries in all (the 500 spheres are just below), the launches run.
 constexpr int REMARK_T = 512;
 template <class L, typename S, bool WALLS, bool B, bool INPLACE>
 __global__ void __launch_bounds__(REMARK_T) k_remark(const RemarkArgs a0, const RemarkArgs* __restrict__ cells)
 {
-    constexpr int CS = B ? REMARK_CLUSTER_BATCH : REMARK_CLUSTER;
     const RemarkArgs& a = B ? cells[blockIdx.y] : a0;
     const int g = (int)blockIdx.x * REMARK_T + (int)threadIdx.x;
-    constexpr int G = CS * REMARK_T;
-    // f(p, e) for the first count(p) entries of every listed particle: the cluster's threads are
-    // split into as many groups of at least 128 as there are particles
-    auto each = [&](const int* list, int n, auto count, auto f) {
-        int groups = 1;
-        while (groups * 2 <= n && groups < G / 128) groups *= 2;
-        const int size = G / groups;
-        for (int b = g / size; b < n; b += groups) {
-            const int p = list[b], m = count(p);
-            for (int e = g % size; e < m; e += size) f(p, e);
-        }
+    const int G = (int)gridDim.x * REMARK_T;  // (the cluster is the grid's x axis)
+    // The cluster's threads split over a list of n particles: particles b, b + groups, ..., and of each
+    // the entries e, e + size, ...
+    struct Part {
+        int b, groups, e, size;
     };
-    auto visited = [&](int p) { return 2 * a.f.pc[p].n_is; };
-    auto all = [&](int p) { return a.f.pc[p].tmpl_n; };
+    auto part = [&](int n) {
+        int groups = 1;
+        while (groups < n && groups < G / 32) groups *= 2;
+        const int size = G / groups;
+        return Part{g / size, groups, g % size, size};
+    };
     const int moved = a.f.cnt ? a.f.cnt->nchanged : 0;  // (a cell of a batch may have no particles)
     if (moved > 0) {
-        if constexpr (!INPLACE) {
-            each(a.f.list, moved, visited, [&](int p, int e) { is_density_entry<L, S>(a.f, p, e); });
-            cluster_barrier<CS>();
-            each(a.f.list, moved, [&](int p) { return a.f.pc[p].n_is; },
-                 [&](int p, int e) { is_restore_entry<L, S, WALLS>(a.f, p, e); });
-            cluster_barrier<CS>();
-        }
-        each(a.f.list, moved, all, [&](int p, int e) { clear_entry(a.p, p, OldAnchor(a.p, p), e); });
-        cluster_barrier<CS>();
         const int restamped = a.f.cnt->nrestamp;
-        each(a.p.restamp, restamped, all, [&](int p, int e) { stamp_entry(a.p, p, e); });
-        cluster_barrier<CS>();
-        each(a.f.list, moved, visited, [&](int p, int e) {
-            if constexpr (INPLACE) inplace_fix_entry<L, S, WALLS>(a.f, p, e);
-            else is_fix_entry<L, S>(a.f, p, e);
+        const Part pm = part(moved), pr = part(restamped);
+        Moved hm{};    // the first particle of each of this thread's lists
+        Stamped hr{};
+        if (pm.b < moved) hm = moved_particle(a.f, a.f.list[pm.b]);
+        auto each_moved = [&](auto f) {
+            for (int b = pm.b; b < moved; b += pm.groups) f(b == pm.b ? hm : moved_particle(a.f, a.f.list[b]));
+        };
+        auto each_restamped = [&](auto f) {
+            for (int b = pr.b; b < restamped; b += pr.groups) f(b == pr.b ? hr : Stamped(a.p.pc, a.p.pk, a.p.restamp[b]));
+        };
+        if constexpr (!INPLACE) {
+            each_moved([&](const Moved& h) {
+                for (int e = pm.e; e < 2 * h.n_is; e += pm.size) is_density_entry<L, S>(a.f, h, e);
+            });
+            cluster_barrier<REMARK_CLUSTER>();
+            each_moved([&](const Moved& h) {
+                for (int e = pm.e; e < h.n_is; e += pm.size) is_restore_entry<L, S, WALLS>(a.f, h, e);
+            });
+            cluster_barrier<REMARK_CLUSTER>();
+        }
+        each_moved([&](const Moved& h) {
+            for (int e = pm.e; e < h.n; e += 4 * pm.size) clear_entries<4>(a.p, h, e, pm.size);
         });
-        each(a.p.restamp, restamped, all, [&](int p, int e) { mask_entry<L>(a.m, p, e); });
+        if (pr.b < restamped) hr = Stamped(a.p.pc, a.p.pk, a.p.restamp[pr.b]);
+        cluster_barrier<REMARK_CLUSTER>();
+        each_restamped([&](const Stamped& h) {
+            for (int e = pr.e; e < h.n; e += 4 * pr.size) stamp_entries<4>(a.p, h, e, pr.size);
+        });
+        cluster_barrier<REMARK_CLUSTER>();
+        each_moved([&](const Moved& h) {
+            for (int e = pm.e; e < 2 * h.n_is; e += pm.size) {
+                if constexpr (INPLACE) inplace_fix_entry<L, S, WALLS>(a.f, h, e);
+                else is_fix_entry<L, S>(a.f, h, e);
+            }
+        });
+        each_restamped([&](const Stamped& h) {
+            for (int e = pr.e; e < h.n; e += pr.size) mask_entry<L>(a.m, h, e);
+        });
     }
     // the streaming of the next pull takes the current wall velocities (k_wall_advance)
     if (a.wv && g < 18) {
@@ -1813,6 +1835,28 @@ inline void launch_cluster(const void* k, dim3 grid, int cluster, int threads, v
     cudaLaunchKernelExC(&c, k, args);
 }
 
+// REMARK_CLUSTER blocks are beyond the portable cluster size: where the device cannot place them
+// (few SMs in each of its groups), the largest portable one.
+inline int remark_cluster(const void* k)
+{
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(REMARK_CLUSTER);
+    c.blockDim = dim3((unsigned)REMARK_T);
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = REMARK_CLUSTER;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, k, &c) == cudaSuccess && n > 0)
+        return REMARK_CLUSTER;
+    cudaGetLastError();
+    return 8;
+}
+
 template <class L, typename S>
 void launch_remark_l(const RemarkArgs& a, const RemarkArgs* cells, int ncells, cudaStream_t s)
 {
@@ -1827,7 +1871,8 @@ void launch_remark_l(const RemarkArgs& a, const RemarkArgs* cells, int ncells, c
     const void* k;
     if (a.f.s.aa) k = walls ? (const void*)k_remark<L, S, true, false, true> : (const void*)k_remark<L, S, false, false, true>;
     else k = walls ? (const void*)k_remark<L, S, true, false, false> : (const void*)k_remark<L, S, false, false, false>;
-    launch_cluster(k, dim3(REMARK_CLUSTER), REMARK_CLUSTER, REMARK_T, args, s);
+    const int cluster = remark_cluster(k);
+    launch_cluster(k, dim3(cluster), cluster, REMARK_T, args, s);
 }
 
 // cells: per-cell arguments of a batch on the device (a's are not read then), or null.
