@@ -308,7 +308,8 @@ int enqueue_step(lbm_ctx* ctx, int c, cudaEvent_t* ev = nullptr)
         sh.max_entries = (long long)ctx->h_tmpl.size();
         launches += launch_particle_phase_a(pa, ctx->stream);
         if (few_entries(sh)) {
-            ctx->kt->remark(ctx->lattice, remark_args(ctx, c), nullptr, 1, ctx->stream);
+            const Geom& g = ctx->g;
+            ctx->kt->remark(ctx->lattice, remark_args(ctx, c), nullptr, 1, g.wall[0] || g.wall[1] || g.wall[2], ctx->stream);
             launches += 1;
             walls_advanced = ctx->moving_walls;
         } else if (ctx->inplace) {

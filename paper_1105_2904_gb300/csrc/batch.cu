@@ -133,11 +133,11 @@ int enqueue_batch_step(lbm_batch* b, int c, cudaEvent_t* ev = nullptr)
         const int nc = (int)b->cells.size();
         launches += launch_particle_phase_batch_a(b->d_part, b->shape, b->stream);
         if (few_entries(b->shape)) {
-            b->kt->remark(b->lattice, RemarkArgs{}, b->d_remark[c], nc, b->stream);
+            b->kt->remark(b->lattice, RemarkArgs{}, b->d_remark[c], nc, b->any_walls, b->stream);
             if (ev) cudaEventRecord(ev[2], b->stream);
             return launches + 1;
         }
-        b->kt->is_save_batch(b->lattice, b->d_isfix[c], nc, b->stream);
+        b->kt->is_save_batch(b->lattice, b->d_isfix[c], nc, b->any_walls, b->stream);
         launches += launch_particle_phase_batch_b(b->d_part, b->shape, b->stream);
         b->kt->is_fix_batch(b->lattice, b->d_isfix[c], nc, b->stream);
         b->kt->update_masks_batch(b->lattice, b->d_mask, nc, b->stream);

@@ -142,7 +142,7 @@ struct KernelTable {
     void (*is_fix)(const ISFixArgs&, cudaStream_t);    // densities into the new IS sites
     int (*sweep_batch)(const BatchSweepArgs&, cudaStream_t);  // returns the kernels launched
     // per-cell argument arrays on the device, blockIdx.y = cell
-    void (*is_save_batch)(int lattice, const ISFixArgs* cells, int ncells, cudaStream_t);
+    void (*is_save_batch)(int lattice, const ISFixArgs* cells, int ncells, bool walls, cudaStream_t);
     void (*is_fix_batch)(int lattice, const ISFixArgs* cells, int ncells, cudaStream_t);
     void (*update_masks_batch)(int lattice, const MaskArgs* cells, int ncells, cudaStream_t);
     void (*features)(const FeatureArgs&, cudaStream_t);
@@ -151,8 +151,8 @@ struct KernelTable {
     // left: 1 after a neighbour phase, 2 after a local phase).
     void (*inplace_fix)(const ISFixArgs&, cudaStream_t);
     // The IS bookkeeping, the owner-map update and the masks in one launch (few_entries); cells:
-    // per-cell arguments on the device, or null.
-    void (*remark)(int lattice, const RemarkArgs&, const RemarkArgs* cells, int ncells, cudaStream_t);
+    // per-cell arguments on the device, or null; walls: the context, or some cell, has them.
+    void (*remark)(int lattice, const RemarkArgs&, const RemarkArgs* cells, int ncells, bool walls, cudaStream_t);
     int elem_bytes;
     int compute_bytes;
 };

@@ -1450,30 +1450,38 @@ __global__ void k_is_density(const ISFixArgs a0, const ISFixArgs* __restrict__ c
 
 // (2) Still before the owner map changes: the sites the sweep saw as IS of a particle whose
 // shift changed get the populations the sweep computed for them (recomputed from the
-// sweep's input with the sweep's particle view; same code, same result bit for bit).
+// sweep's input with the sweep's particle view; same code, same result bit for bit). One copy of the
+// machine code for every kernel that restores: inlined into each, the compiler chose other products to
+// fuse in some of them, and a walled FP32 or BF16 cell of a batch, or a 2D box with few particles, came
+// out an FP32 rounding away from the same cell stepped alone or with more particles.
 template <class L, typename S, bool WALLS>
-__device__ __forceinline__ void is_restore_entry(const ISFixArgs& a, const Moved& h, int e)
+__device__ __noinline__ void restore_site(const SweepArgs& a, unsigned site, unsigned t)
 {
     using C = typename Store<S>::C;
-    const Geom& g = a.s.g;
-    unsigned site;
-    if (!visited_site(a, h, e, site)) return;  // (e < n_is: at the old anchor)
-    const unsigned t = a.s.pv.tag[site];
-    if (t != ((CLS_IS << 30) | (unsigned)h.p)) return;
+    const Geom& g = a.g;
     const int x = (int)(site % (unsigned)g.nx);
     const int y = (int)((site / (unsigned)g.nx) % (unsigned)g.ny);
     const int z = (int)(site / ((unsigned)g.nx * (unsigned)g.ny));
     const Nbr n = neighbours<WALLS>(g, x, y, z);
     C f[L::Q];
-    pull<L, S, WALLS>((const S*)a.s.fin, g, n, x, y, z, site, f);
+    pull<L, S, WALLS>((const S*)a.fin, g, n, x, y, z, site, f);
     // (FP64 storage: the input already holds the imposed values, k_impose_plain)
-    sweep_site<L, S, WALLS, Store<S>::deviation, true>(a.s, x, y, z, site, true, n, f, t, a.s.pv.ismask[site]);
+    sweep_site<L, S, WALLS, Store<S>::deviation, true>(a, x, y, z, site, true, n, f, t, a.pv.ismask[site]);
+}
+
+template <class L, typename S, bool WALLS>
+__device__ __forceinline__ void is_restore_entry(const ISFixArgs& a, const Moved& h, int e)
+{
+    unsigned site;
+    if (!visited_site(a, h, e, site)) return;  // (e < n_is: at the old anchor)
+    const unsigned t = a.s.pv.tag[site];
+    if (t == ((CLS_IS << 30) | (unsigned)h.p)) restore_site<L, S, WALLS>(a.s, site, t);
 }
 
 template <class L, typename S, bool WALLS, bool B>
-__global__ void k_is_restore(const ISFixArgs a0, const ISFixArgs* __restrict__ cells)
+__global__ void k_is_restore(const __grid_constant__ ISFixArgs a0, const ISFixArgs* __restrict__ cells)
 {
-    const ISFixArgs a = pick_args<B>(a0, cells);
+    const ISFixArgs& a = B ? cells[blockIdx.y] : a0;
     if (!a.cnt) return;
     const int nlist = a.cnt->nchanged;
     for (int b = blockIdx.x; b < nlist; b += gridDim.x) {
@@ -1577,7 +1585,7 @@ __global__ void k_inplace_fix(const ISFixArgs a)
 // template entries in all (the 500 spheres are just below), the launches run.
 constexpr int REMARK_T = 512;
 template <class L, typename S, bool WALLS, bool B, bool INPLACE>
-__global__ void __launch_bounds__(REMARK_T) k_remark(const RemarkArgs a0, const RemarkArgs* __restrict__ cells)
+__global__ void __launch_bounds__(REMARK_T, 1) k_remark(const __grid_constant__ RemarkArgs a0, const RemarkArgs* __restrict__ cells)
 {
     const RemarkArgs& a = B ? cells[blockIdx.y] : a0;
     const int g = (int)blockIdx.x * REMARK_T + (int)threadIdx.x;
@@ -1858,16 +1866,15 @@ inline int remark_cluster(const void* k)
 }
 
 template <class L, typename S>
-void launch_remark_l(const RemarkArgs& a, const RemarkArgs* cells, int ncells, cudaStream_t s)
+void launch_remark_l(const RemarkArgs& a, const RemarkArgs* cells, int ncells, bool walls, cudaStream_t s)
 {
     RemarkArgs arg = a;
     void* args[2] = {&arg, &cells};
     if (cells) {
-        launch_cluster((const void*)k_remark<L, S, true, true, false>, dim3(REMARK_CLUSTER_BATCH, ncells),
-                       REMARK_CLUSTER_BATCH, REMARK_T, args, s);
+        launch_cluster(walls ? (const void*)k_remark<L, S, true, true, false> : (const void*)k_remark<L, S, false, true, false>,
+                       dim3(REMARK_CLUSTER_BATCH, ncells), REMARK_CLUSTER_BATCH, REMARK_T, args, s);
         return;
     }
-    const bool walls = a.f.s.g.wall[0] || a.f.s.g.wall[1] || a.f.s.g.wall[2];
     const void* k;
     if (a.f.s.aa) k = walls ? (const void*)k_remark<L, S, true, false, true> : (const void*)k_remark<L, S, false, false, true>;
     else k = walls ? (const void*)k_remark<L, S, true, false, false> : (const void*)k_remark<L, S, false, false, false>;
@@ -1875,12 +1882,13 @@ void launch_remark_l(const RemarkArgs& a, const RemarkArgs* cells, int ncells, c
     launch_cluster(k, dim3(cluster), cluster, REMARK_T, args, s);
 }
 
-// cells: per-cell arguments of a batch on the device (a's are not read then), or null.
+// cells: per-cell arguments of a batch on the device (a's are not read then), or null. walls: the
+// context, or some cell, has them.
 template <typename S>
-void launch_remark(int lattice, const RemarkArgs& a, const RemarkArgs* cells, int ncells, cudaStream_t s)
+void launch_remark(int lattice, const RemarkArgs& a, const RemarkArgs* cells, int ncells, bool walls, cudaStream_t s)
 {
-    if (lattice == 0) launch_remark_l<D2Q9, S>(a, cells, ncells, s);
-    else launch_remark_l<D3Q19, S>(a, cells, ncells, s);
+    if (lattice == 0) launch_remark_l<D2Q9, S>(a, cells, ncells, walls, s);
+    else launch_remark_l<D3Q19, S>(a, cells, ncells, walls, s);
 }
 
 template <typename S>
@@ -1892,11 +1900,11 @@ void launch_update_masks(const MaskArgs& a, cudaStream_t s)
 
 // Batched forms (one lattice for every cell of a batch; walls: some cell has them).
 template <typename S>
-void launch_is_save_batch(int lattice, const ISFixArgs* cells, int nc, cudaStream_t s)
+void launch_is_save_batch(int lattice, const ISFixArgs* cells, int nc, bool walls, cudaStream_t s)
 {
     const dim3 grid(std::max(2, 256 / nc), nc);
-    if (lattice == 0) launch_is_save_l<D2Q9, S, true>(ISFixArgs{}, cells, grid, true, s);
-    else launch_is_save_l<D3Q19, S, true>(ISFixArgs{}, cells, grid, true, s);
+    if (lattice == 0) launch_is_save_l<D2Q9, S, true>(ISFixArgs{}, cells, grid, walls, s);
+    else launch_is_save_l<D3Q19, S, true>(ISFixArgs{}, cells, grid, walls, s);
 }
 
 template <typename S>
