@@ -224,6 +224,7 @@ lbm_status build(lbm_batch* b)
     b->moving.clear();
     b->shape = PhaseShape{};
     b->shape.ncells = nc;
+    b->shape.batch = 1;
     b->shape.scratch_f64 = b->precision == LBM_FP64 ? 1 : 0;
     long long max_pairs = 1;
     for (int i = 0; i < nc; ++i) {

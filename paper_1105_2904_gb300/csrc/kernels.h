@@ -252,6 +252,7 @@ struct PhaseShape {
     int pair_cap;     // contact-pair capacity of every cell (its resolve buffer)
     int scratch_f64;  // FP64 storage: ordered per-particle sums
     long long max_entries;  // template entries of the cell with the most
+    int batch;        // 1: the cells of a batch
 };
 // The shape of a single context (max_entries is the caller's to set).
 PhaseShape phase_shape(const ParticleArgs& a);

@@ -700,8 +700,11 @@ __global__ void k_stamp_all(const ParticleArgs a)
 // Particle phase of a step: 64^3 suspension (31 spheres) 73 -> 26 us, 64-cell ensemble 88 -> 36 us.
 // At 2000 particles k_contacts_move takes 35 us, as long as the six launches it replaces (8 SMs'
 // FP64 pipes move all particles), so from FEW_MAX_P on, and for contact grids of more than
-// FEW_MAX_C cells (shared memory), the per-phase kernels above run.
-constexpr int FEW_T = 512, FEW_CLUSTER = 8, FEW_MAX_P = 1024, FEW_MAX_C = 8192;
+// FEW_MAX_C cells (shared memory), the per-phase kernels above run. A cell of a batch has one block
+// instead of a cluster, so the line lies at fewer particles: a step of 8 cells with 100, 200, 300 and
+// 500 spheres of radius 4 each takes 112, 184, 269 and 436 us in this form and 124, 193, 266 and 402 us
+// in launches, of 32 cells with 200 615 and 618 us, of 4 cells with 1000 of radius 3 308 and 216 us.
+constexpr int FEW_T = 512, FEW_CLUSTER = 8, FEW_MAX_P = 1024, FEW_MAX_P_BATCH = 256, FEW_MAX_C = 8192;
 
 template <bool B, bool F64>
 __global__ void __launch_bounds__(RT) k_sums_accel(const ParticleArgs a0, const ParticleArgs* __restrict__ cells)
@@ -941,7 +944,10 @@ PhaseShape phase_shape(const ParticleArgs& a)
     return sh;
 }
 
-bool few_particles(const PhaseShape& sh) { return sh.max_np <= FEW_MAX_P && sh.max_cells <= FEW_MAX_C; }
+bool few_particles(const PhaseShape& sh)
+{
+    return sh.max_np <= (sh.batch ? FEW_MAX_P_BATCH : FEW_MAX_P) && sh.max_cells <= FEW_MAX_C;
+}
 
 int launch_particle_phase_a(const ParticleArgs& a, cudaStream_t s)
 {

@@ -104,3 +104,15 @@ def test_above_the_limits_matches_oracle(case, streaming, precision, bar_u, bar_
         assert np.max(np.abs(g.get_particles()["force"] - fo)) <= bar_f * np.max(np.abs(fo))
     assert np.any(before != o.get_tags())
     g.close()
+
+
+# A cell of a batch has one block for its contacts where a single context has a cluster, so the
+# launches per phase take over at fewer particles (measured: between 200 and 300 a cell).
+@pytest.mark.parametrize("n,few", [(256, True), (257, False)])
+def test_batch_of_many_particles_a_cell_takes_the_launches_per_phase(n, few):
+    parts = _particles(O.D3Q19, (57, 60, 62), n, 2.0, (0, 0, 0), 5)
+    b = lbmp.Batch(O.D3Q19, [(57, 60, 62), (20, 20, 20)], [0.8] * 2, [(0.0, 0.0, 0.0)] * 2, precision="fp32", gap=0.3)
+    b.add_particles(0, *parts)
+    # sweep, sums, contacts and re-marking; or the sweep and at least one launch per phase
+    assert (b.info()["launches_per_step"] == 4) == few
+    b.close()
