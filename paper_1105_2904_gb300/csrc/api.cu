@@ -229,6 +229,7 @@ SweepArgs sweep_args(lbm_ctx* ctx, int c)
     a.bs_scratch = ctx->bs_scratch;
     a.pc = ctx->pc;
     a.tmpl = ctx->tmpl;
+    a.entries = (long long)ctx->h_tmpl.size();
     a.omega = 1.0 / ctx->tau;
     a.pre = 1.0 - 0.5 / ctx->tau;
     for (int k = 0; k < 3; ++k) a.F[k] = ctx->F[k];

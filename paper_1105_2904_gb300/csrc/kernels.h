@@ -26,6 +26,7 @@ struct SweepArgs {
     float omega_f, pre_f, F_f[3];  // the same in FP32 (reduced-storage sweeps)
     int moving_walls;          // 1: wall faces may move (uw is read)
     const WallVel* uw;         // wall velocities of the streaming that the pull completes
+    long long entries;         // template entries of all particles
     int ahead;                 // k_sweep2: groups of rows to prefetch ahead (0: none)
     int pair_bx;               // deviation storage, even nx: two-site kernel with this many
                                // threads along x (16, 32, 64 or 128); 0: one-site kernel
@@ -128,6 +129,28 @@ struct FeatureArgs {
     double u_ref;              // velocity scale
     float* out;                // [np][n_side^3][4]
 };
+
+// Groups of `by` rows that the FP32 two-site sweep with bx threads along x prefetches ahead (k_sweep2),
+// 0 for none. Rows of the populations brought into L2 some PREFETCH_SITES sites ahead of the blocks in
+// flight shorten the wait for DRAM of a sweep that its particles hold up; a sweep without particles
+// already runs at the copy rate and only loses L2 to them. Sweep us without and with prefetch, particles
+// of radius 8 in a share of the sites:
+//   share 0.256: 128^3 62.7, 61.9; 256^3 436, 424; 512 x 64 x 128 116.7, 112.8; 512^3 3515, 3479
+//   share 0.08:  128^3 56.6, 56.3; 512 x 64 x 128 106.1, 104.5; 256^3 399, 402; 512^3 3192, 3300; so up to
+//                2^23 sites only (2D, 1024 x 2048 with 0.075: 35.5, 34.3)
+//   none:        130 x 128 x 128 61.4, 62.4; 512^3 2984, 3123; 8192 x 32 x 32 188, 244; 2D 2048 x 512, which
+//                stays in L2, 10.5, 13.3
+// Groups of fewer than 512 sites (64 x 512 x 256, share 0.256: 223, 227) and of more than 16384 (one
+// thread's prefetch of a long row; 4096 x 64 x 64 with 0.256 453, 445, 2D 32768 x 512 without particles
+// 177, 191) and wider blocks (256^3, bx = 64: 451, 465) do without.
+constexpr long long PREFETCH_SITES = 131072, PREFETCH_MIN_SITES = 1ll << 20;
+inline int prefetch_groups(const Geom& g, long long entries, int bx, int by)
+{
+    const long long N = g.N, group = (long long)g.nx * by;
+    if (bx != 16 || N < PREFETCH_MIN_SITES || group < 512 || group > 16384) return 0;
+    if (entries * (N <= (1ll << 23) ? 16 : 8) < N) return 0;
+    return (int)(PREFETCH_SITES / group) + 1;
+}
 
 struct RemarkArgs;
 

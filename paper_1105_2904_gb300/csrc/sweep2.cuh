@@ -467,14 +467,6 @@ __device__ __forceinline__ void bs_transfer_dev2(const SweepArgs& a, int x0, int
     if (bs1) sc[1] = make_float4(dv[0].y, dv[1].y, dv[2].y, __uint_as_float(tags.y));
 }
 
-// FP32 storage: rows of the populations brought into L2 ahead of the blocks in flight, some
-// PREFETCH_SITES sites (one bulk prefetch per direction and group of rows, by the group's first
-// block), shorten the wait for DRAM and are read in long bursts: 256^3 suspension 0.438 -> 0.424
-// ms, 512^3 3.52 -> 3.50 ms. Further ahead they are evicted before use (two and five times the
-// distance: 0.509 and 0.584 ms). The 16-bit sweep gains nothing (3.16 -> 3.20 ms), and boxes that
-// stay in L2 from step to step have no use for it.
-constexpr unsigned PREFETCH_SITES = 131072, PREFETCH_MIN_SITES = 1u << 20;
-
 // One block: BX threads along x (2 BX sites) times 64 / BX rows of one z-plane (one row for BX = 128),
 // twenty warps per SM (96 registers; twenty-four with spills were slower). Blocks of two warps
 // instead of four leave fewer slots waiting for a block's last warp: 512^3 FP32 3.523 -> 3.491 ms,
@@ -494,7 +486,8 @@ __global__ void __launch_bounds__(pair_threads(BX), 640 / pair_threads(BX)) k_sw
     const bool valid = xr < g.nx && yr < g.ny;
     const int x0 = min(xr, g.nx - 2), y = min(yr, g.ny - 1);
     const unsigned idx = ((unsigned)z * (unsigned)g.ny + (unsigned)y) * (unsigned)g.nx + (unsigned)x0;
-    if (sizeof(S) == 4 && blockIdx.x == 0 && a.ahead && threadIdx.x < Q) {
+    // (one bulk prefetch per direction and group of rows, by the group's first block; prefetch_groups)
+    if (sizeof(S) == 4 && PART && BX == 16 && blockIdx.x == 0 && a.ahead && threadIdx.x < Q) {
         unsigned gy = blockIdx.y + (unsigned)a.ahead;
         const unsigned zz = blockIdx.z + gy / gridDim.y;
         gy %= gridDim.y;
@@ -623,7 +616,7 @@ template <class L, typename S, bool WALLS, bool PART>
 void launch_sweep2_v(SweepArgs a, int bx, cudaStream_t s)
 {
     const int threads = pair_threads(bx), by = threads / bx;
-    a.ahead = a.g.N >= PREFETCH_MIN_SITES ? (int)(PREFETCH_SITES / ((unsigned)a.g.nx * (unsigned)by)) + 1 : 0;
+    a.ahead = sizeof(S) == 4 && PART ? prefetch_groups(a.g, a.entries, bx, by) : 0;
     const dim3 grid((a.g.nx + 2 * bx - 1) / (2 * bx), (a.g.ny + by - 1) / by, a.g.nz);
     switch (bx) {
     case 16: k_sweep2<L, S, WALLS, PART, 16><<<grid, threads, 0, s>>>(a); break;
