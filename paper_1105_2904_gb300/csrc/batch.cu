@@ -37,6 +37,7 @@ struct lbm_batch {
     int4* d_table = nullptr;
     int ntiles = 0;             // of the schedule (lbm_schedule_tiles)
     int launch_tiles = 0;       // of d_table (sweep_tiles)
+    bool flat = false;          // some of them in index order
     PhaseShape shape{};
     bool any_part = false, any_walls = false;
     std::vector<int> moving;  // cells with moving walls
@@ -123,6 +124,7 @@ int enqueue_batch_step(lbm_batch* b, int c, cudaEvent_t* ev = nullptr)
     a.ncells = (int)b->cells.size();
     a.table = b->d_table;
     a.ntiles = b->launch_tiles;
+    a.flat = b->flat ? 1 : 0;
     a.walls = b->any_walls ? 1 : 0;
     a.part = b->any_part ? 1 : 0;
     a.grid = b->grid;
@@ -280,6 +282,7 @@ lbm_status build(lbm_batch* b)
     if (table.size() >= (1ull << 31)) return bfail(b, LBM_E_INVALID, "too many tiles");
     b->ntiles = (int)nt;
     b->launch_tiles = (int)table.size();
+    b->flat = std::any_of(table.begin(), table.end(), [](const int4& t) { return t.z < 0; });
     const bool few = few_entries(b->shape);
     for (int c = 0; c < 2; ++c) {
         BS(upload(b, &b->d_sweep[c], sw[c]));

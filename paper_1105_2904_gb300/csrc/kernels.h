@@ -113,6 +113,7 @@ struct BatchSweepArgs {
     int ncells;
     const int4* table;         // device [ntiles]
     int ntiles;
+    int flat;                  // some tiles are in index order
     int walls;                 // some cell has walls
     int part;                  // some cell has particles
     int grid;                  // 0: one block per tile; > 0: that many blocks stride over the table

@@ -1117,8 +1117,9 @@ __global__ void __launch_bounds__(SWEEP_THREADS, Store<S>::deviation ? 9 : 1) k_
 // stride of them in the persistent form) and runs the same per-site step as k_sweep with the
 // arguments of the tile's cell. Deviation storages without walls are held to nine blocks per SM
 // (56 registers, a few bytes of spills): eight and ten blocks 0.971 and 1.112 ms against 0.958 ms at
-// the 64-cell ensemble.
-template <class L, typename S, bool WALLS, bool PART>
+// the 64-cell ensemble. FLAT: some tiles of the table are runs in index order; a table without any does
+// without the choice (8 cells of 128^3, FP16: 345 -> 334 us).
+template <class L, typename S, bool WALLS, bool PART, bool FLAT>
 __global__ void __launch_bounds__(SWEEP_THREADS, (Store<S>::deviation && !WALLS) ? 9 : 1)
     k_sweep_batch(const BatchSweepArgs b)
 {
@@ -1143,7 +1144,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS, (Store<S>::deviation && !WALLS)
         int x, y, z;
         bool valid;
         unsigned idx;
-        if (Store<S>::deviation && t.z < 0) {  // 128 sites in index order from t.y on
+        if (FLAT && t.z < 0) {  // 128 sites in index order from t.y on
             const unsigned at = (unsigned)t.y + threadIdx.x;
             valid = at < g.N;
             idx = min(at, g.N - 1u);
@@ -1927,7 +1928,13 @@ template <class L, typename S, bool WALLS, bool PART>
 void launch_sweep_batch_v(const BatchSweepArgs& b, cudaStream_t s)
 {
     const unsigned grid = b.grid > 0 ? (unsigned)b.grid : (unsigned)b.ntiles;
-    k_sweep_batch<L, S, WALLS, PART><<<grid, SWEEP_THREADS, 0, s>>>(b);
+    if constexpr (Store<S>::deviation) {
+        if (b.flat) {
+            k_sweep_batch<L, S, WALLS, PART, true><<<grid, SWEEP_THREADS, 0, s>>>(b);
+            return;
+        }
+    }
+    k_sweep_batch<L, S, WALLS, PART, false><<<grid, SWEEP_THREADS, 0, s>>>(b);
 }
 
 template <class L, typename S>
