@@ -272,7 +272,11 @@ constexpr int UPD_THREADS = 128;
 constexpr int KCHUNK = 9;            // k-steps of weights a warp loads at once (the closure's 17 in two)
 constexpr int RCHUNK = 8;            // k-steps of rows a warp of k_update loads at once (128 rows)
 constexpr int SPLITS = 16;           // fixed-order split of the rows in the weight gradients
-// Up to here a 16-row block's pass over all weights (512 kB from L2) stays a matter of a few us.
+constexpr int LOSS_TILES = 4;        // sums of 256 squared errors per warp of k_update
+// Up to here a 16-row block's pass over all weights (512 kB from L2) stays a matter of a few us, and the
+// fused form is the faster one at every number of rows: gradients through 256-512-256, 262144 weights,
+// fused and layer by layer, 128 rows 68 and 261 us, 1024 156 and 369, 16384 1771 and 2504, 65536 6960
+// and 9550; through 64-256-256-64 45 and 257, 67 and 291, 503 and 1216, 1932 and 4208.
 constexpr long long FUSED_WEIGHTS = 262144;
 constexpr size_t FUSED_SMEM = 160 * 1024;
 
@@ -327,6 +331,8 @@ struct UpdateArgs {
     float lr, b1, b2, eps;
     double* loss;        // loss of the minibatch is added here
     double loss_scale;
+    float* loss_part;    // sums of the squared errors of 256 outputs each (more than LOSS_TILES of them)
+    int* loss_done;      // loss warps that are through, zero between launches
 };
 
 // C (16 rows of `in` times a K x N operand in fragment order, plus the bias if given) for this
@@ -611,16 +617,52 @@ __global__ void __launch_bounds__(UPD_THREADS) k_update(const UpdateArgs a)
         }
         return;
     }
-    if (task == 0) {
-        const long long m = (long long)a.rows * n.size[n.L];
-        double tot = 0.0;
-        for (long long b = 0; b < m; b += 256) {
-            float x[8];
+    // The loss: sums of 256 squared errors, LOSS_TILES of them to a warp, added in order by the warp
+    // that is through last (by the only one where there is one). One warp for all of them took 0.8 us
+    // for each sum: gradients of 16384 rows through 64-256-256-64 2.12 -> 0.50 ms (layer by layer 1.22 ms).
+    const long long m = (long long)a.rows * n.size[n.L];
+    const int tiles = (int)((m + 255) / 256), warps = (tiles + LOSS_TILES - 1) / LOSS_TILES;
+    if (task >= warps) return;
+    float s[LOSS_TILES];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) x[j] = b + lane + 32 * j < m ? n.r2[b + lane + 32 * j] : 0.f;
-            tot += (double)tree256(x);
-        }
+    for (int k = 0; k < LOSS_TILES; ++k) {
+        const long long b = ((long long)task * LOSS_TILES + k) * 256 + lane;
+        float x[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = b + 32 * j < m ? n.r2[b + 32 * j] : 0.f;
+        s[k] = tree256(x);
+    }
+    double tot = 0.0;
+    if (warps == 1) {
+#pragma unroll
+        for (int k = 0; k < LOSS_TILES; ++k)
+            if (k < tiles) tot += (double)s[k];
         if (lane == 0) *a.loss += tot * a.loss_scale;
+        return;
+    }
+    int last = 0;
+    if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < LOSS_TILES; ++k)
+            if (task * LOSS_TILES + k < tiles) a.loss_part[task * LOSS_TILES + k] = s[k];
+        __threadfence();
+        last = atomicAdd(a.loss_done, 1) == warps - 1;
+    }
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();
+    float next = lane < tiles ? __ldcg(&a.loss_part[lane]) : 0.f;
+    for (int b = 0; b < tiles; b += 32) {
+        const float v = next;
+        next = b + 32 + lane < tiles ? __ldcg(&a.loss_part[b + 32 + lane]) : 0.f;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+            const float t = __shfl_sync(0xffffffffu, v, k);
+            if (b + k < tiles) tot += (double)t;
+        }
+    }
+    if (lane == 0) {
+        *a.loss += tot * a.loss_scale;
+        *a.loss_done = 0;
     }
 }
 
@@ -688,6 +730,8 @@ struct lbm_mlp {
     __nv_bfloat16* wb = nullptr;     // and backwards
     std::vector<__nv_bfloat16*> hT, dT;
     float* r2 = nullptr;
+    float* loss_part = nullptr;
+    int* loss_done = nullptr;
     std::vector<void*> allocs;
     std::string err;
 };
@@ -748,8 +792,9 @@ lbm_status ensure_rows(lbm_mlp* net, int rows)
         for (auto* q : net->hT) free_dev(net, q);
         for (auto* q : net->dT) free_dev(net, q);
         free_dev(net, net->r2);
+        free_dev(net, net->loss_part);
         net->cap = 0;
-        net->r2 = nullptr;
+        net->r2 = net->loss_part = nullptr;
         net->hT.assign(net->L, nullptr);
         net->dT.assign(net->L, nullptr);
         for (size_t l = 0; l < (size_t)net->L; ++l) {
@@ -757,6 +802,7 @@ lbm_status ensure_rows(lbm_mlp* net, int rows)
             if ((s = malloc_dev(net, &net->dT[l], (size_t)cap * net->sizes[l + 1])) != LBM_OK) return s;
         }
         if ((s = malloc_dev(net, &net->r2, (size_t)cap * O)) != LBM_OK) return s;
+        if ((s = malloc_dev(net, &net->loss_part, ((size_t)cap * O + 255) / 256)) != LBM_OK) return s;
         net->cap = cap;
         return LBM_OK;
     }
@@ -915,8 +961,11 @@ void fused_update(lbm_mlp* net, int rows, int slot, bool step, float lr, float b
     a.b2 = b2;
     a.eps = eps;
     a.loss = net->loss_dev + slot;
-    a.loss_scale = 1.0 / (double)((long long)rows * net->sizes[(size_t)net->L]);
-    int tasks = 1;
+    const long long outputs = (long long)rows * net->sizes[(size_t)net->L];
+    a.loss_scale = 1.0 / (double)outputs;
+    a.loss_part = net->loss_part;
+    a.loss_done = net->loss_done;
+    int tasks = (int)((outputs + 256 * LOSS_TILES - 1) / (256 * LOSS_TILES));
     for (size_t l = 0; l < (size_t)net->L; ++l)
         tasks += (net->sizes[l + 1] + 15) / 16 * ((net->sizes[l] + 7) / 8) + net->sizes[l + 1];
     constexpr int W = UPD_THREADS / 32;
@@ -994,7 +1043,9 @@ lbm_status lbm_mlp_create(lbm_mlp** out, int nlayers, const int* sizes, void* cu
     net->fused = weights <= FUSED_WEIGHTS && rows_smem(net, true) <= FUSED_SMEM &&
                  cudaFuncSetAttribute(k_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM) == cudaSuccess;
     if (net->fused)
-        s = (s = malloc_dev(net, &net->wf, (size_t)wf)) != LBM_OK ? s : malloc_dev(net, &net->wb, (size_t)wb);
+        s = (s = malloc_dev(net, &net->wf, (size_t)wf)) != LBM_OK || (s = malloc_dev(net, &net->wb, (size_t)wb)) != LBM_OK
+                ? s
+                : malloc_dev(net, &net->loss_done, 1);
     else
         s = malloc_dev(net, &net->p16, (size_t)off);
     if (s != LBM_OK) {
@@ -1004,6 +1055,7 @@ lbm_status lbm_mlp_create(lbm_mlp** out, int nlayers, const int* sizes, void* cu
     if (net->fused) {  // the fragments' padding stays zero
         cudaMemsetAsync(net->wf, 0, sizeof(__nv_bfloat16) * wf, net->stream);
         cudaMemsetAsync(net->wb, 0, sizeof(__nv_bfloat16) * wb, net->stream);
+        cudaMemsetAsync(net->loss_done, 0, sizeof(int), net->stream);
     } else {
         cudaMemsetAsync(net->p16, 0, sizeof(__nv_bfloat16) * off, net->stream);
     }
