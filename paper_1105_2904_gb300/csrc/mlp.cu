@@ -447,7 +447,11 @@ __global__ void __launch_bounds__(ROWS_THREADS) k_rows(const RowsArgs a)
             __nv_bfloat16* out = h[l + 1];
             const int ldo = tile_ld(N);
             rows_gemm(h[l], tile_ld(K), K, N, n.wf + n.wf_off[l], bias,
-                      [&](int r, int c, float v) { out[r * ldo + c] = __float2bfloat16(fmaxf(v, 0.f)); });
+                      [&](int r, int c, float v) {
+                          // (rows beyond the last stay zero: k_update multiplies them by zero gradients, and
+                          // relu(bias ...) of a zero input can be infinite where no real row's is)
+                          out[r * ldo + c] = __float2bfloat16(row0 + r < a.rows ? fmaxf(v, 0.f) : 0.f);
+                      });
         } else {
             rows_gemm(h[l], tile_ld(K), K, N, n.wf + n.wf_off[l], bias, [&](int r, int c, float y) {
                 if (row0 + r >= a.rows) return;
