@@ -219,7 +219,8 @@ lbm_status lbm_profile_steps(lbm_ctx* ctx, int n, double out_ms[3]);
  * 4-byte accesses and packed FP32 pair arithmetic; blocks of 64 threads, 128 for threads_x =
  * 128, threads_x of them along x); 0 selects the one-site kernel; -1 (the default) picks
  * the two-site kernel with 16 threads along x (the one-site kernel where nx is odd). FP64
- * storage always uses the one-site kernel. Drops the captured step graphs. LBM_E_INVALID for
+ * storage has one form whatever the shape: with the pull scheme three kernels (imposition, sweep,
+ * particle sites) of one site per thread, in place the one-site kernel. Drops the captured step graphs. LBM_E_INVALID for
  * other values. */
 lbm_status lbm_set_sweep_shape(lbm_ctx* ctx, int threads_x);
 
@@ -342,8 +343,8 @@ lbm_status lbm_bs_exchange_noalloc(int lattice, int nx, int ny, int nz, const in
  * launch over all cells (a schedule table of 128-thread tiles, each tile one rectangle of
  * one x-y plane of one cell; cells whose tiles would leave over a tenth of their threads idle
  * are swept in index order, 128 consecutive sites a tile) and one launch per particle-phase
- * kernel (the cell as the second grid index; FP64 storage three for the sweep), captured in CUDA graphs of one or several steps. Each cell's result
- * is bit for bit the result of stepping it alone with the one-site sweep kernel
+ * kernel (the cell as the second grid index; FP64 storage three for the sweep), captured in CUDA
+ * graphs of one or several steps. Each cell's result is bit for bit the result of stepping it alone with the one-site sweep kernel
  * (lbm_set_sweep_shape(ctx, 0)); the batch sweep is that kernel. */
 
 /* Creates ncells contexts sharing the lattice, storage precision, face kinds, particle
@@ -370,7 +371,8 @@ lbm_ctx* lbm_batch_cell(lbm_batch* b, int cell);
 
 /* Launch tuning (results do not depend on it):
  *   tile_width[ncells]: sites along x of a cell's tiles, 32, 64 or 128 (the tile then spans
- *     128/width rows in y); NULL = 128 for every cell;
+ *     128/width rows in y); NULL = 128 for every cell. FP32 / FP16 / BF16 cells that these tiles
+ *     fill to less than nine tenths are swept in index order instead, whatever their width;
  *   order: 0 cells one after another, 1 one tile of each cell in turn, 2 largest cell first;
  *   grid: 0 = one block per tile, > 0 = that many resident blocks striding over the table;
  *   steps_per_graph: steps captured in one graph launch (1..256).
@@ -386,8 +388,8 @@ lbm_status lbm_batch_synchronize(lbm_batch* b);
 /* As lbm_profile_steps, for the whole batch: out_ms = mean sweep, particle phase, step. */
 lbm_status lbm_batch_profile_steps(lbm_batch* b, int n, double out_ms[3]);
 
-/* out[0] cells, out[1] lattice sites of all cells, out[2] particles, out[3] sweep tiles,
- * out[4] kernels launched per step. Captures the step graphs if needed. */
+/* out[0] cells, out[1] lattice sites of all cells, out[2] particles, out[3] tiles of the
+ * schedule (lbm_schedule_tiles, before cells take index order), out[4] kernels launched per step. Captures the step graphs if needed. */
 lbm_status lbm_batch_get_info(lbm_batch* b, long long out[5]);
 
 /* The cudaStream_t every cell of the batch enqueues on. */
@@ -396,7 +398,9 @@ void* lbm_batch_stream(lbm_batch* b);
 /* Host-only (no device needed): the sweep schedule of a batch. Returns the number of tiles
  * for ncells cells of sizes dims[ncells*3] with tile_width[ncells] (NULL = 128) in the given
  * order (as lbm_batch_set_tuning), or -1 on a bad argument. If out != NULL it receives 4
- * ints per tile in launch order: cell, x0, y0 | (log2(width) << 16), z. */
+ * ints per tile in launch order: cell, x0, y0 | (log2(width) << 16), z. This is the schedule of
+ * row tiles; in the launch a cell that is swept in index order (lbm_batch_set_tuning) has
+ * ceil(sites / 128) tiles of 128 consecutive sites in their place. */
 long long lbm_schedule_tiles(int ncells, const int* dims, const int* tile_width, int order, int* out);
 
 /* Description of the last non-OK status of b (never NULL). */

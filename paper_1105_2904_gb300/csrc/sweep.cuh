@@ -11,13 +11,15 @@
 // replaced by f^eq_d(rho_I, u_p + omega_p x r), with rho_I the post-collision density of
 // that site. Only sites inside a particle can pull from an IS site (every neighbour of an IS
 // site lies in the particle), so fluid sites never look. This removes a separate scattered
-// pass over the IS shell.
+// pass over the IS shell. (FP64 storage with the pull scheme, bound by the FP64 pipe instead of
+// memory, does make that pass: k_impose_plain writes the imposed values into `fin` before the
+// sweep, which is thus modified by its own step.)
 //
 // Density carry: since no pull uses the populations of an IS site raw, the sweep stores an
 // IS site's post-collision density rho_I in all Q of its slots instead. The value a site
 // pulls from an IS source is then rho_I itself: the imposition needs no second, dependent
 // load. The particle phase keeps this true when site sets move (k_is_density, k_is_restore,
-// k_is_fix).
+// k_is_fix, or k_remark in their place).
 //
 // In-place streaming (SweepArgs::aa, one buffer): two kinds of step alternate. From the
 // natural layout (slot i of x holds f*_i(x)) the neighbour phase pulls as above and writes
@@ -1125,7 +1127,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS, (Store<S>::deviation && !WALLS)
 {
     using C = typename Store<S>::C;
     constexpr int Q = L::Q;
-    // The tile's cell arguments (~190 bytes) are staged in shared memory by the block and
+    // The tile's cell arguments (sizeof(SweepArgs)) are staged in shared memory by the block and
     // reloaded only when the cell changes, instead of every thread loading them per tile.
     __shared__ __align__(16) SweepArgs sa;
     int cur = -1;
@@ -1574,9 +1576,9 @@ __global__ void k_inplace_fix(const ISFixArgs a)
 // ---- few template entries: the whole re-marking in one launch ---------------------------------
 // The kernels above and the owner-map update between them are six launches of 2.5 us that find
 // nothing to do in most steps of a small suspension (a sphere at u = 1e-3 crosses a site boundary
-// once in some 300 steps). Here they are one: a cluster of 16 blocks returns at once when no shift
-// changed, and otherwise spreads each moved particle's entries over its 8192 threads with a
-// cluster barrier where the launches had a boundary. In a fast suspension every phase has work for
+// once in some 300 steps). Here they are one: a cluster of 16 blocks (8 for few entries) returns at once
+// when no shift changed, and otherwise spreads each moved particle's entries over its 8192 threads with
+// a cluster barrier where the launches had a boundary. In a fast suspension every phase has work for
 // more threads than a cluster has, and what counts is the chain of loads per entry: the particle's
 // record and anchors are loaded once for all phases and entries, four entries are cleared or stamped
 // at a time. The five phases of a step that moves 90 of 800 disks of radius 10 take 28 us (a cluster
@@ -1659,8 +1661,6 @@ __global__ void __launch_bounds__(REMARK_T, 1) k_remark(const __grid_constant__ 
 namespace lbmp {
 
 // ---- launchers --------------------------------------------------------------------------
-// Deviation storages with an even nx take the two-site kernel (a.pair_bx threads along x),
-// everything else the one-site kernel.
 // FP64 storage, pull scheme: returns the launches made.
 template <class L>
 int launch_sweep_plain(const SweepArgs& a, cudaStream_t s)
@@ -1675,6 +1675,8 @@ int launch_sweep_plain(const SweepArgs& a, cudaStream_t s)
     return part ? 3 : 1;
 }
 
+// Reduced storages, pull scheme: the two-site kernel for even nx (a.pair_bx threads along x), else the
+// one-site kernel.
 template <class L, typename S, bool WALLS, bool PART>
 void launch_sweep_v(const SweepArgs& a, cudaStream_t s)
 {
