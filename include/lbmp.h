@@ -220,8 +220,8 @@ lbm_status lbm_profile_steps(lbm_ctx* ctx, int n, double out_ms[3]);
  * 128, threads_x of them along x); 0 selects the one-site kernel; -1 (the default) picks
  * the two-site kernel with 16 threads along x (the one-site kernel where nx is odd). FP64
  * storage has one form whatever the shape: with the pull scheme three kernels (imposition, sweep,
- * particle sites) of one site per thread, in place the one-site kernel. Drops the captured step graphs. LBM_E_INVALID for
- * other values. */
+ * particle sites) of one site per thread, in place the one-site kernel. Drops the captured step
+ * graphs. LBM_E_INVALID for other values. */
 lbm_status lbm_set_sweep_shape(lbm_ctx* ctx, int threads_x);
 
 /* Streaming scheme (no counterpart in the paper, whose Eq. 4 only states that f*_i(x) moves
