@@ -505,7 +505,7 @@ __device__ __forceinline__ bool pull_bounces(const Nbr& n)
     }
 }
 
-template <class L, bool WALLS>
+template <class L, bool WALLS, bool CHECKED = true>
 __device__ __forceinline__ void substitute_is_other_dev(const Geom& g, const Nbr& n, int x, int y, int z, unsigned owner,
                                                      const PartView& pv, float f[]);
 
@@ -516,7 +516,8 @@ __device__ __forceinline__ void substitute_is_other_dev(const Geom& g, const Nbr
 // directions some lane of the warp needs are evaluated by every lane and kept where the
 // lane's own mask asks for them (no per-lane branches, no loads beyond the owner's record).
 // Every lane of the warp that is converged here calls it; m = 0 for sites with nothing to do.
-template <class L, bool WALLS>
+// CHECKED = false: the caller has checked the owners (bounds-checked build).
+template <class L, bool WALLS, bool CHECKED = true>
 __device__ __forceinline__ void substitute_is_dev(const Geom& g, const Nbr& n, int x, int y, int z,
                                                   unsigned m, unsigned owner, const PartView& pv, float f[])
 {
@@ -525,7 +526,7 @@ __device__ __forceinline__ void substitute_is_dev(const Geom& g, const Nbr& n, i
     const unsigned wm = __reduce_or_sync(__activemask(), mm);
     if (wm) {
         unsigned ow = mm ? owner : 0u;
-        if (!LBM_DCHECK(pv.status, ow < (unsigned)pv.np)) ow = 0u;
+        if (CHECKED && !LBM_DCHECK(pv.status, ow < (unsigned)pv.np)) ow = 0u;
         const PKernF k = pv.pkf[ow];
         float r[3], ux[3];
         lever_arm(g, k, x, y, z, r);
@@ -575,12 +576,12 @@ __device__ __forceinline__ void substitute_is_dev(const Geom& g, const Nbr& n, i
             }
         });
     }
-    if (m & MASK_OTHER) substitute_is_other_dev<L, WALLS>(g, n, x, y, z, owner, pv, f);
+    if (m & MASK_OTHER) substitute_is_other_dev<L, WALLS, CHECKED>(g, n, x, y, z, owner, pv, f);
 }
 
 // Sources owned by another particle than the site's own (site sets of close particles
 // meet): rare, one direction at a time.
-template <class L, bool WALLS>
+template <class L, bool WALLS, bool CHECKED>
 __device__ __forceinline__ void substitute_is_other_dev(const Geom& g, const Nbr& n, int x, int y, int z, unsigned owner,
                                                      const PartView& pv, float f[])
 {
@@ -600,7 +601,7 @@ __device__ __forceinline__ void substitute_is_other_dev(const Geom& g, const Nbr
             const unsigned sidx = ((unsigned)sz * (unsigned)g.ny + (unsigned)sy) * (unsigned)g.nx + (unsigned)sx;
             const unsigned t = pv.tag[sidx];
             if ((t >> 30) != CLS_IS || (t & PID_MASK) == owner) continue;
-            if (!LBM_DCHECK(pv.status, (t & PID_MASK) < (unsigned)pv.np)) continue;
+            if (CHECKED && !LBM_DCHECK(pv.status, (t & PID_MASK) < (unsigned)pv.np)) continue;
             const PKernF k = pv.pkf[t & PID_MASK];
             float r[3], us[3];
             lever_arm(g, k, sx, sy, sz, r);
@@ -767,7 +768,7 @@ __device__ __forceinline__ void sweep_site(const SweepArgs& a, int x, int y, int
             if constexpr (AA != 0)
                 is_density_from_array_warp<L, C, WALLS>(g, n, x, y, z, idx, m, a.pv, (const C*)a.is_rho_in, f);
             if constexpr (St::deviation)
-                substitute_is_dev<L, WALLS>(g, n, x, y, z, m, tagx & PID_MASK, a.pv, f);
+                substitute_is_dev<L, WALLS, !RESTORE>(g, n, x, y, z, m, tagx & PID_MASK, a.pv, f);
             else if (m)
                 substitute_is_plain<L, WALLS>(g, n, x, y, z, idx, m, a.pv, f);
         }
@@ -792,7 +793,7 @@ __device__ __forceinline__ void sweep_site(const SweepArgs& a, int x, int y, int
         // Particle-fluid momentum transfer at BS sites (Eqs. 5-7).
         const bool isbs = valid && (tagx >> 30) == CLS_BS;
         if constexpr (St::deviation) {
-            if (isbs)
+            if (!RESTORE && isbs)  // (only IS sites are restored)
                 bs_transfer_dev<L, std::is_same<S, float>::value>(a, x, y, z, idx, tagx, mrho, mj0, mj1, mj2, f);
         } else if (isbs && LBM_DCHECK(a.pv.status, (tagx & PID_MASK) < (unsigned)a.pv.np)) {
             C r[3], ub[3], ubp[3], du[3];
@@ -1456,7 +1457,8 @@ __global__ void k_is_density(const ISFixArgs a0, const ISFixArgs* __restrict__ c
 // sweep's input with the sweep's particle view; same code, same result bit for bit). One copy of the
 // machine code for every kernel that restores: inlined into each, the compiler chose other products to
 // fuse in some of them, and a walled FP32 or BF16 cell of a batch, or a 2D box with few particles, came
-// out an FP32 rounding away from the same cell stepped alone or with more particles.
+// out an FP32 rounding away from the same cell stepped alone or with more particles. For the same reason
+// the checks of the bounds-checked build are made by the caller (sources_known).
 template <class L, typename S, bool WALLS>
 __device__ __noinline__ void restore_site(const SweepArgs& a, unsigned site, unsigned t)
 {
@@ -1472,13 +1474,37 @@ __device__ __noinline__ void restore_site(const SweepArgs& a, unsigned site, uns
     sweep_site<L, S, WALLS, Store<S>::deviation, true>(a, x, y, z, site, true, n, f, t, a.pv.ismask[site]);
 }
 
+// Bounds-checked build: the owners of the IS sites that site pulls from are particles.
+template <class L, bool WALLS>
+__device__ __forceinline__ bool sources_known(const SweepArgs& a, unsigned site)
+{
+    bool known = true;
+#ifdef LBM_DEBUG
+    const Geom& g = a.g;
+    const int x = (int)(site % (unsigned)g.nx);
+    const int y = (int)((site / (unsigned)g.nx) % (unsigned)g.ny);
+    const int z = (int)(site / ((unsigned)g.nx * (unsigned)g.ny));
+    const Nbr n = neighbours<WALLS>(g, x, y, z);
+    sfor<0, L::Q>([&](auto ic) {
+        constexpr int i = decltype(ic)::value;
+        int sx, sy, sz;
+        unsigned sidx;
+        bool bounce;
+        pull_source<L, i, WALLS>(g, n, x, y, z, site, sx, sy, sz, sidx, bounce);
+        const unsigned t = a.pv.tag[sidx];
+        if ((t >> 30) == CLS_IS) known = known && LBM_DCHECK(a.pv.status, (t & PID_MASK) < (unsigned)a.pv.np);
+    });
+#endif
+    return known;
+}
+
 template <class L, typename S, bool WALLS>
 __device__ __forceinline__ void is_restore_entry(const ISFixArgs& a, const Moved& h, int e)
 {
     unsigned site;
     if (!visited_site(a, h, e, site)) return;  // (e < n_is: at the old anchor)
     const unsigned t = a.s.pv.tag[site];
-    if (t == ((CLS_IS << 30) | (unsigned)h.p)) restore_site<L, S, WALLS>(a.s, site, t);
+    if (t == ((CLS_IS << 30) | (unsigned)h.p) && sources_known<L, WALLS>(a.s, site)) restore_site<L, S, WALLS>(a.s, site, t);
 }
 
 template <class L, typename S, bool WALLS, bool B>
