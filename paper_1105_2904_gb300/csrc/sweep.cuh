@@ -918,8 +918,12 @@ __device__ __forceinline__ void sweep_site(const SweepArgs& a, int x, int y, int
 // The site of a thread of the one-site kernels, and whether it is the thread's to work on (a thread
 // beyond the end takes a site it never stores). Rows: 128-site tiles of one row (block x, y, z). FLAT:
 // sites in index order, which leaves no lane idle whatever the row length and costs the divisions
-// that find the coordinates.
-template <bool FLAT>
+// that find the coordinates. SELECT: the coordinate of a thread beyond the end by a select instead of a
+// min; the same value, but the kernels around it come out faster with one or the other: in place in 2D
+// SELECT (4096 x 2048 FP16 walled 113 -> 106 us), in place in 3D min (384^3 FP32 with particles 1694 ->
+// 1663 us), pull in FP32, 2D, or without walls and particles SELECT (2D 4095 x 4096 FP16 160.1 -> 157.0
+// us), else min (255 x 254 x 253 FP16 walled 354 -> 338 us, with particles 405 -> 401 us).
+template <bool FLAT, bool SELECT>
 __device__ __forceinline__ bool one_site(const Geom& g, int& x, int& y, int& z, unsigned& idx)
 {
     if constexpr (FLAT) {
@@ -935,9 +939,8 @@ __device__ __forceinline__ bool one_site(const Geom& g, int& x, int& y, int& z, 
         z = blockIdx.z;
         const unsigned row = ((unsigned)z * (unsigned)g.ny + (unsigned)y) * (unsigned)g.nx;
         const int xr = blockIdx.x * SWEEP_THREADS + threadIdx.x;
-        // (the select, not min(xr, nx - 1): 16-bit rows 1 to 7 % faster, 4095 x 4096 FP16 160.1 -> 157.0 us)
         const bool valid = xr < g.nx;
-        x = valid ? xr : g.nx - 1;
+        x = SELECT ? (valid ? xr : g.nx - 1) : min(xr, g.nx - 1);
         idx = row + (unsigned)x;
         return valid;
     }
@@ -963,7 +966,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS, WALLS ? (FLAT ? 7 : 1) : 9) k_s
     const Geom& g = a.g;
     int x, y, z;
     unsigned idx;
-    const bool valid = one_site<FLAT>(g, x, y, z, idx);
+    const bool valid = one_site<FLAT, sizeof(S) == 4 || L::D == 2 || (!WALLS && !PART)>(g, x, y, z, idx);
     const Nbr n = neighbours<WALLS>(g, x, y, z);
     // Owner tag and IS-source mask are loaded with the populations (no dependent round trip).
     unsigned tagx = TAG_FLUID, mask = 0;
@@ -1095,7 +1098,7 @@ __global__ void __launch_bounds__(SWEEP_THREADS, Store<S>::deviation ? 9 : 1) k_
     const Geom& g = a.g;
     int x, y, z;
     unsigned idx;
-    const bool valid = one_site<FLAT>(g, x, y, z, idx);
+    const bool valid = one_site<FLAT, L::D == 2>(g, x, y, z, idx);
     const Nbr n = neighbours<WALLS>(g, x, y, z);
     unsigned tagx = TAG_FLUID, mask = 0;
     if constexpr (PART) {
